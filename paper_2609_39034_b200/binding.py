@@ -1,8 +1,10 @@
-"""Thin ctypes binding of libswila.so: argument marshalling only.
+"""Thin binding of libswila.so: argument marshalling only.
 
 Every step of the recurrence runs inside the CUDA library; this module turns torch
-tensors into raw device pointers and mirrors the C structs of include/swila.h.  There
-is no CPU fallback: importing this module raises if the library has not been built."""
+tensors into raw device pointers and mirrors the C structs of include/swila.h.  The calls a
+program makes per token or per layer go through a small C++ module (_swila_torch), the rest
+through ctypes.  There is no CPU fallback: importing this module raises if the library has not
+been built."""
 from __future__ import annotations
 
 import ctypes
@@ -119,6 +121,7 @@ def _load() -> ctypes.CDLL:
 
 
 lib = _load()
+from . import _swila_torch as _ext  # noqa: E402  (linked against the library that has just been loaded)
 
 
 def make_shape(w: Workload, T: Optional[int] = None, algo: int = ALGO_AUTO) -> Shape:
@@ -173,15 +176,11 @@ def swila_forward(w: Workload, inp: dict, *, state_in: Optional[dict] = None, st
     include/swila.h).  state_in / state_out: dicts with W (and r_prev, rho_prev when
     TEMPORAL), or None (initial state / discard).  Returns o."""
     T = inp["q"].shape[2] if T is None else T
-    sh = make_shape(w, T=T, algo=algo)
     if o is None:
         o = torch.empty((w.B, w.H, T, w.Dv), device=inp["q"].device, dtype=w.torch_io_dtype)
-    g = _gates(inp)
-    sin = _state(state_in["W"], state_in.get("r_prev"), state_in.get("rho_prev")) if state_in else None
-    sout = _state(state_out["W"], state_out.get("r_prev"), state_out.get("rho_prev")) if state_out else None
-    check(lib.swila_forward(ctypes.byref(sh), _p(inp["q"]), _p(inp["k"]), _p(inp["v"]), ctypes.byref(g),
-                            ctypes.byref(sin) if sin else None, ctypes.byref(sout) if sout else None,
-                            _p(o), _p(r_debug), _stream(stream)))
+    rc = _ext.forward(w, inp, state_in, state_out, o, r_debug, None, algo, stream, T)
+    if rc:
+        raise SwilaError(rc)
     return o
 
 
@@ -199,37 +198,31 @@ def swila_forward_stats(w: Workload, inp: dict, stats: dict, *, state_in: Option
     """swila_forward that also ADDS the sums over time of the mixture weights (Sec. 3.5) to the
     buffers in ``stats`` (keys r_sum, r_ent, rho_sum, rho_ent; a missing key or None skips that sum)."""
     T = inp["q"].shape[2] if T is None else T
-    sh = make_shape(w, T=T, algo=algo)
     if o is None:
         o = torch.empty((w.B, w.H, T, w.Dv), device=inp["q"].device, dtype=w.torch_io_dtype)
-    g = _gates(inp)
-    sin = _state(state_in["W"], state_in.get("r_prev"), state_in.get("rho_prev")) if state_in else None
-    sout = _state(state_out["W"], state_out.get("r_prev"), state_out.get("rho_prev")) if state_out else None
-    st = Stats(*[(_p(stats.get(n)) or ctypes.c_void_p(None)).value for n in ("r_sum", "r_ent", "rho_sum", "rho_ent")])
-    check(lib.swila_forward_stats(ctypes.byref(sh), _p(inp["q"]), _p(inp["k"]), _p(inp["v"]), ctypes.byref(g),
-                                  ctypes.byref(sin) if sin else None, ctypes.byref(sout) if sout else None,
-                                  _p(o), _p(r_debug), ctypes.byref(st), _stream(stream)))
+    rc = _ext.forward(w, inp, state_in, state_out, o, r_debug, stats, algo, stream, T)
+    if rc:
+        raise SwilaError(rc)
     return o
 
 
 def swila_output_norm(w: Workload, o: torch.Tensor, weight: Optional[torch.Tensor] = None, eps: float = 1e-6,
                       stream=None) -> torch.Tensor:
     """RMSNorm of o [B,H,T,Dv] over its last axis, in place (App. D.1); weight fp32 [Dv] or None."""
-    sh = make_shape(w, T=o.shape[2])
-    check(lib.swila_output_norm(ctypes.byref(sh), _p(o), _p(weight), ctypes.c_float(eps), _stream(stream)))
+    rc = _ext.norm(w, o, weight, eps, stream, o.shape[2])
+    if rc:
+        raise SwilaError(rc)
     return o
 
 
 def swila_decode_step(w: Workload, inp: dict, state: dict, *, o: Optional[torch.Tensor] = None,
                       algo: int = ALGO_AUTO, stream=None) -> torch.Tensor:
     """One token on a carried state (updated in place).  Returns o [B,H,1,Dv]."""
-    sh = make_shape(w, T=1, algo=algo)
     if o is None:
         o = torch.empty((w.B, w.H, 1, w.Dv), device=inp["q"].device, dtype=w.torch_io_dtype)
-    g = _gates(inp)
-    st = _state(state["W"], state.get("r_prev"), state.get("rho_prev"))
-    check(lib.swila_decode_step(ctypes.byref(sh), _p(inp["q"]), _p(inp["k"]), _p(inp["v"]), ctypes.byref(g),
-                                ctypes.byref(st), _p(o), _stream(stream)))
+    rc = _ext.decode(w, inp, state, o, algo, stream)
+    if rc:
+        raise SwilaError(rc)
     return o
 
 

@@ -16,6 +16,8 @@ CSRC = os.path.join(HERE, "csrc")
 INC = os.path.join(os.path.dirname(HERE), "include")
 OBJ = os.path.join(HERE, "build")
 LIB = os.path.join(HERE, "libswila.so")
+EXT = os.path.join(HERE, "_swila_torch.so")  # marshalling of torch tensors, linked against LIB
+EXT_SRC = os.path.join(CSRC, "swila_torch.cpp")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
@@ -71,20 +73,52 @@ def _compile(unit, verbose):
     return out, r.stderr
 
 
+def _build_ext(force: bool) -> None:
+    """The marshalling module: plain C++ against the headers of this interpreter and of torch."""
+    import sysconfig
+
+    import torch
+    from torch.utils import cpp_extension as ce
+
+    h = hashlib.sha256((torch.__version__ + sys.version).encode())
+    for f in sorted(_deps(EXT_SRC)):
+        h.update(open(f, "rb").read())
+    stamp_file = os.path.join(OBJ, "ext.stamp")
+    if not force and os.path.exists(EXT) and os.path.exists(stamp_file) and open(stamp_file).read() == h.hexdigest():
+        return
+    cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
+    tmp = EXT + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include")]
+    for d in ce.include_paths():
+        cmd += ["-isystem", d]
+    cmd += [EXT_SRC, "-o", tmp, "-L", HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"]
+    for d in ce.library_paths():
+        cmd += ["-L", d]
+    cmd += ["-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"building {os.path.basename(EXT)} failed:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, EXT)
+    with open(stamp_file, "w") as f:
+        f.write(h.hexdigest())
+
+
 def build(force: bool = False, verbose: bool = False, jobs: int | None = None) -> str:
     """Compile what changed (an object is rebuilt when its source, a file it includes or the flags change) and link."""
     os.makedirs(OBJ, exist_ok=True)
     units = _units()
     stamps = {u[0]: _unit_stamp(u) for u in units}
+    link_stamp = hashlib.sha256("".join(sorted(stamps.values())).encode()).hexdigest()
+    link_file = os.path.join(OBJ, "stamp")
+    if not force and os.path.exists(LIB) and os.path.exists(link_file) and open(link_file).read() == link_stamp:
+        _build_ext(force)
+        return LIB  # also where only the library was brought along, without the objects it was linked from
     stale = []
     for u in units:
         sf = os.path.join(OBJ, u[0] + ".stamp")
         if force or not os.path.exists(os.path.join(OBJ, u[0])) or not os.path.exists(sf) or open(sf).read() != stamps[u[0]]:
             stale.append(u)
-    link_stamp = hashlib.sha256("".join(sorted(stamps.values())).encode()).hexdigest()
-    link_file = os.path.join(OBJ, "stamp")
-    if not stale and os.path.exists(LIB) and os.path.exists(link_file) and open(link_file).read() == link_stamp:
-        return LIB
     logs = []
     if stale:
         jobs = jobs or min(len(stale), os.cpu_count() or 4)
@@ -103,6 +137,7 @@ def build(force: bool = False, verbose: bool = False, jobs: int | None = None) -
         f.write(link_stamp)
     if verbose:
         sys.stderr.write("\n".join(logs))
+    _build_ext(force)
     return LIB
 
 

@@ -93,7 +93,7 @@ static bool chunk_covers(const swila_shape_t *s, bool aux) {
 
 static int run(const swila_shape_t *s, int T, const void *q, const void *k, const void *v, const swila_gates_t *g,
                const swila_state_t *sin, swila_state_t *sout, void *o, float *r_debug, void *stream,
-               const swila_stats_t *stats = nullptr) {
+               const swila_stats_t *stats = nullptr, long long heads = 0) {
   const bool temporal = (s->flags & SWILA_TEMPORAL) != 0;
   const bool gated = (s->flags & SWILA_GATED) != 0;
   if (!q || !k || !v || !g || !o) return SWILA_ERR_NULL;
@@ -165,6 +165,7 @@ static int run(const swila_shape_t *s, int T, const void *q, const void *k, cons
     a.p.r_sum = stats->r_sum; a.p.r_ent = stats->r_ent;
     a.p.rho_sum = stats->rho_sum; a.p.rho_ent = stats->rho_ent;
   }
+  a.heads = heads > 0 ? heads : (long long)s->B * s->H;
   a.Dk = s->Dk; a.J = s->J; a.io_dtype = s->io_dtype;
   a.gate_mode = !gated ? 0 : (s->gate_granularity == SWILA_GATE_PER_KEY ? 1 : s->gate_granularity == SWILA_GATE_ELEMENTWISE ? 3 : 2);
   a.post = (s->flags & SWILA_POST_DECAY) ? 1 : 0;
@@ -213,6 +214,9 @@ __global__ void fill_kernel(float *p, size_t n, float val) {
 
 using namespace swila;
 
+static int forward_any(const swila_shape_t *s, const void *q, const void *k, const void *v, const swila_gates_t *g,
+                       const swila_state_t *state_in, swila_state_t *state_out, void *o, float *r_debug, void *stream, long long heads);
+
 extern "C" {
 
 int swila_version(void) { return 200; }
@@ -248,7 +252,7 @@ int swila_device_status(void) {
     if (e != cudaSuccess) return cuda_fail(e);
   }
   if (flag) {  // (warp + 1) << 16 | low half of the barrier's shared-memory address; 1 if only a hand-over flag gave up
-    snprintf(g_cuda_err, sizeof(g_cuda_err), "a bounded wait expired inside the chunked kernel (warp %d, barrier at 0x%x)",
+    snprintf(g_cuda_err, sizeof(g_cuda_err), "a bounded wait expired inside a kernel (warp %d, barrier at 0x%x)",
              (flag >> 16) - 1, flag & 0xffff);
     return SWILA_ERR_CUDA;
   }
@@ -280,6 +284,14 @@ int swila_state_init(const swila_shape_t *s, swila_state_t *st, void *stream) {
 
 int swila_forward(const swila_shape_t *s, const void *q, const void *k, const void *v, const swila_gates_t *g,
                   const swila_state_t *state_in, swila_state_t *state_out, void *o, float *r_debug, void *stream) {
+  return forward_any(s, q, k, v, g, state_in, state_out, o, r_debug, stream, 0);
+}
+
+}  // extern "C"
+
+// heads: (batch, head) pairs of the problem this call is a slab of (0: it is the whole problem)
+static int forward_any(const swila_shape_t *s, const void *q, const void *k, const void *v, const swila_gates_t *g,
+                       const swila_state_t *state_in, swila_state_t *state_out, void *o, float *r_debug, void *stream, long long heads) {
   int rc = check_shape(s, true);
   if (rc) return rc;
   if (s->T == 0) {  // nothing to scan: the state passes through
@@ -299,8 +311,10 @@ int swila_forward(const swila_shape_t *s, const void *q, const void *k, const vo
       e = cudaMemcpyAsync(state_out->rho_prev, state_in->rho_prev, r_elems(s) * 4, cudaMemcpyDeviceToDevice, cs);
     return e == cudaSuccess ? SWILA_OK : cuda_fail(e);
   }
-  return run(s, s->T, q, k, v, g, state_in, state_out, o, r_debug, stream);
+  return run(s, s->T, q, k, v, g, state_in, state_out, o, r_debug, stream, nullptr, heads);
 }
+
+extern "C" {
 
 int swila_forward_stats(const swila_shape_t *s, const void *q, const void *k, const void *v, const swila_gates_t *g,
                         const swila_state_t *state_in, swila_state_t *state_out, void *o, float *r_debug,
@@ -472,8 +486,8 @@ int swila_forward_host(const swila_shape_t *s, const void *q, const void *k, con
     swila_gates_t dg = {ws + h.beta + lo(h.n_gate), ws + h.pik + lo(h.n_gate), ws + h.piq + lo(h.n_gate),
                         temporal ? ws + h.gk + lo(h.n_tg) : nullptr, temporal ? ws + h.gq + lo(h.n_tg) : nullptr,
                         gated ? (const float *)(ws + h.alpha + lo(h.n_alpha)) : nullptr};
-    rc = swila_forward(&sub, ws + h.q + lo(h.n_qk), ws + h.k + lo(h.n_qk), ws + h.v + lo(h.n_v), &dg,
-                       state_in ? &dstate : nullptr, state_out ? &dstate : nullptr, ws + h.o + lo(h.n_v), nullptr, stream);
+    rc = forward_any(&sub, ws + h.q + lo(h.n_qk), ws + h.k + lo(h.n_qk), ws + h.v + lo(h.n_v), &dg,
+                       state_in ? &dstate : nullptr, state_out ? &dstate : nullptr, ws + h.o + lo(h.n_v), nullptr, stream, nbh);
     if (rc) return rc;
     if (hp) {
       e = cudaEventRecord(hp->computed[i], cs);

@@ -54,7 +54,6 @@
 // and the sums over time behind the load-balancing loss of Sec. 3.5.
 #pragma once
 
-#include <cuda.h>  // CUtensorMap and its enums (types only; the encoder is fetched through the runtime)
 #include <cuda_bf16.h>
 
 #include <atomic>
@@ -62,6 +61,7 @@
 
 #include "swila_chunk_sched.h"
 #include "swila_common.cuh"
+#include "swila_tma_maps.h"
 #include "swila_umma.cuh"
 
 namespace swila {
@@ -1377,34 +1377,6 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
   if (warp == 8) tmem_dealloc(*tmem_base_s, Cf::TM_ALLOC);
 }
 
-// cuTensorMapEncodeTiled, fetched through the runtime so that the library does not link against the driver.
-typedef CUresult (*ChunkEncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
-                                       const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
-                                       CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-inline ChunkEncodeTiledFn chunk_encode_fn() {
-  static ChunkEncodeTiledFn fn = [] {
-    void *sym = nullptr;
-    cudaDriverEntryPointQueryResult res;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &sym, cudaEnableDefault, &res) != cudaSuccess ||
-        res != cudaDriverEntryPointSuccess)
-      sym = nullptr;
-    return (ChunkEncodeTiledFn)sym;
-  }();
-  return fn;
-}
-
-// One bf16 tensor map: `rank` dimensions (innermost first) of sizes `dims` with byte strides `strides` (for dimensions
-// 1 .. rank-1) and a copy box of `box` elements; no swizzle, out-of-range elements read as zero.
-inline bool chunk_encode(CUtensorMap *map, const void *base, int rank, const cuuint64_t *dims, const cuuint64_t *strides,
-                         const cuuint32_t *box, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE) {
-  ChunkEncodeTiledFn fn = chunk_encode_fn();
-  if (!fn) return false;
-  const cuuint32_t ones[4] = {1, 1, 1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, (cuuint32_t)rank, const_cast<void *>(base), dims, strides, box, ones,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // Tensor maps of one launch.  k, q [BH][T][DK] as (DK, T, BH) with a box of 64 key dims x 32 tokens and the 128-byte
 // swizzle, which is how the operand tile stores them; v [BH][T][Dv] as (Dv, T, BH); the gate
 // logits [BH][T][J][Dv] as (Dv, J, T, BH) with a box of GROW columns, all J components, 32 tokens.
@@ -1415,17 +1387,17 @@ bool chunk_make_maps(const ScanParams &p, ChunkMaps *m) {
     const cuuint64_t dims[3] = {DK, T, BH};
     const cuuint64_t strides[2] = {DK * 2, T * DK * 2};
     const cuuint32_t box[3] = {64, (cuuint32_t)Cf::C, 1};
-    if (!chunk_encode(&m->k, p.k, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !chunk_encode(&m->q, p.q, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
+    if (!tma_encode(&m->k, p.k, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !tma_encode(&m->q, p.q, 3, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
       return false;
   }
   {
     const cuuint64_t dims[3] = {Dv, T, BH};
     const cuuint64_t strides[2] = {Dv * 2, T * Dv * 2};
     const cuuint32_t box[3] = {(cuuint32_t)Cf::COLS, (cuuint32_t)Cf::C, 1};
-    if (!chunk_encode(&m->v, p.v, 3, dims, strides, box)) return false;
+    if (!tma_encode(&m->v, p.v, 3, dims, strides, box)) return false;
     if constexpr (Cf::TEMPORAL) {
-      if (!chunk_encode(&m->gk, p.gk_logit, 3, dims, strides, box) || !chunk_encode(&m->gq, p.gq_logit, 3, dims, strides, box))
+      if (!tma_encode(&m->gk, p.gk_logit, 3, dims, strides, box) || !tma_encode(&m->gq, p.gq_logit, 3, dims, strides, box))
         return false;
     }
   }
@@ -1433,19 +1405,11 @@ bool chunk_make_maps(const ScanParams &p, ChunkMaps *m) {
     const cuuint64_t dims[4] = {Dv, J, T, BH};
     const cuuint64_t strides[3] = {Dv * 2, J * Dv * 2, T * J * Dv * 2};
     const cuuint32_t box[4] = {(cuuint32_t)Cf::GROW, (cuuint32_t)Cf::J, (cuuint32_t)Cf::C, 1};
-    if (!chunk_encode(&m->be, p.beta_logit, 4, dims, strides, box) || !chunk_encode(&m->pk, p.pik_logit, 4, dims, strides, box) ||
-        !chunk_encode(&m->pq, p.piq_logit, 4, dims, strides, box))
+    if (!tma_encode(&m->be, p.beta_logit, 4, dims, strides, box) || !tma_encode(&m->pk, p.pik_logit, 4, dims, strides, box) ||
+        !tma_encode(&m->pq, p.piq_logit, 4, dims, strides, box))
       return false;
   }
   return true;
-}
-
-// Number of SMs of the current device (one block is resident per SM).
-inline int chunk_sm_count() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  return n;
 }
 
 // Launch counter shared by every instantiation: the value a launch publishes in the hand-over flags
@@ -1467,7 +1431,8 @@ int launch_chunk(const LaunchArgs &a) {
   if constexpr (!GATED && J <= 8) {
     if (aux) kern = swila_chunk_kernel<Cf, true>;
   }
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM_BYTES);
+  static std::atomic<uint64_t> granted[2];
+  cudaError_t e = allow_smem((const void *)kern, Cf::SMEM_BYTES, granted[aux]);
   if (e != cudaSuccess) return (int)e;
   const long long nslice = (a.p.Dv + Cf::COLS - 1) / Cf::COLS;
   const long long ntiles = nslice * a.p.B * a.p.H;
@@ -1482,11 +1447,14 @@ int launch_chunk(const LaunchArgs &a) {
   // tiles, so that the last wave is not half empty (chunk_plan).  The state of a split tile travels through the
   // state output, hence only when that is given; blocks of such a launch wait for each other, hence the
   // cooperative launch (all blocks resident or no launch at all).
-  const ChunkPlan pl = chunk_plan((long long)a.p.B * a.p.H, nslice, nch, chunk_sm_count(),
+  const ChunkPlan pl = chunk_plan((long long)a.p.B * a.p.H, nslice, nch, sm_count(),
                                    a.p.W_out != nullptr && (!TEMPORAL || (a.p.r_out && a.p.rho_out)), kChunkFlagTiles);
   if (pl.split) {
-    unsigned *flags = nullptr;
-    if (cudaGetSymbolAddress((void **)&flags, g_chunk_flags) == cudaSuccess) {
+    static std::atomic<unsigned *> flags_of[kMaxDevices];
+    const int dev = current_device();
+    unsigned *flags = dev >= 0 ? flags_of[dev].load(std::memory_order_relaxed) : nullptr;
+    if (!flags && cudaGetSymbolAddress((void **)&flags, g_chunk_flags) == cudaSuccess && dev >= 0) flags_of[dev].store(flags, std::memory_order_relaxed);
+    if (flags) {
       const unsigned epoch = chunk_next_epoch();
       ChunkSched ss{(int)pl.units, pl.nch, pl.per, pl.gang, epoch, flags + (size_t)(epoch % kChunkFlagSlots) * kChunkFlagTiles};
       void *args[] = {(void *)&prm, (void *)&ss, (void *)&maps};

@@ -72,9 +72,15 @@ int chunk_gated_dispatch(LaunchArgs &a) {
   if (!((a.J == 4 && (a.Dk == 64 || a.Dk == 128)) || (a.J == 8 && a.Dk == 64))) return -1000;
   if (a.p.r_debug || a.p.r_sum || a.p.r_ent || a.p.rho_sum || a.p.rho_ent) return -1000;
   static std::atomic<unsigned> counter{0};
-  unsigned *flags = nullptr;
-  cudaError_t e = cudaGetSymbolAddress((void **)&flags, g_gate_guard);
-  if (e != cudaSuccess) return (int)e;
+  static std::atomic<unsigned *> flags_of[kMaxDevices];
+  const int dev = current_device();
+  unsigned *flags = dev >= 0 ? flags_of[dev].load(std::memory_order_relaxed) : nullptr;
+  cudaError_t e = cudaSuccess;
+  if (!flags) {
+    e = cudaGetSymbolAddress((void **)&flags, g_gate_guard);
+    if (e != cudaSuccess) return (int)e;
+    if (dev >= 0) flags_of[dev].store(flags, std::memory_order_relaxed);
+  }
   unsigned *flag = flags + (counter++ % kGuardSlots);
   e = cudaMemsetAsync(flag, 0, sizeof(unsigned), a.stream);
   if (e != cudaSuccess) return (int)e;

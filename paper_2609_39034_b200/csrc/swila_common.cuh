@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/swila.h"
 
 namespace swila {
@@ -37,14 +39,44 @@ constexpr float kL2Eps = 1e-6f;
 
 struct LaunchArgs {
   ScanParams p;
+  long long heads;  // (batch, head) pairs of the whole problem, of which this launch may be a slab: what sizes are judged by
   int Dk, J, io_dtype, gate_mode /*0 none, 1 per-key, 2 per-row, 3 per-element*/, post, algo;
   cudaStream_t stream;
 };
+
+// What a launch needs to know about the current device, asked of the runtime once per device: every runtime call is a
+// good part of a microsecond, and a decode step is a few.  Several threads may find the same value at the same time.
+constexpr int kMaxDevices = 64;
+inline int current_device() {  // -1: unknown, ask the runtime for everything
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < kMaxDevices ? dev : -1;
+}
+inline int sm_count() {
+  static std::atomic<int> known[kMaxDevices];
+  const int dev = current_device();
+  int n = dev >= 0 ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (n) return n;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev >= 0 ? dev : 0) != cudaSuccess) return 0;
+  if (dev >= 0) known[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
+// Dynamic shared memory above the default limit has to be asked for, once per kernel and device; `granted` is the kernel's own word.
+inline cudaError_t allow_smem(const void *kern, int bytes, std::atomic<uint64_t> &granted) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  const int dev = current_device();
+  if (dev >= 0 && (granted.load(std::memory_order_relaxed) >> dev & 1)) return cudaSuccess;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && dev >= 0) granted.fetch_or(1ull << dev, std::memory_order_relaxed);
+  return e;
+}
 
 // Dispatch entry of one translation unit (one key dimension, one gate mode).
 // Returns SWILA_OK, SWILA_ERR_UNSUPPORTED or SWILA_ERR_CUDA.
 template <int DK, int GATE, bool POST>
 int scan_dispatch(const LaunchArgs &a);
+// Likewise for the blocked scan; err: the device word an expired wait leaves its code in.
+template <int DK, int GATE>
+int block_dispatch(const LaunchArgs &a, int *err, int sms);
 
 // ---------------------------------------------------------------------------------------
 constexpr float kLog2e = 1.4426950408889634f;
@@ -76,6 +108,11 @@ __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 __device__ __forceinline__ void from_f32(float &dst, float x) { dst = x; }
 __device__ __forceinline__ void from_f32(__nv_bfloat16 &dst, float x) { dst = __float2bfloat16_rn(x); }
+
+// Programmatic dependent launch: wait until the launches before this one in the stream are complete and visible (nothing of
+// global memory may be touched earlier), and let the next launch's blocks be set up while this one still runs.
+__device__ __forceinline__ void launch_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // 16-byte asynchronous global->shared copy, L2 only; src_bytes == 0 zero-fills.
 __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src, int src_bytes) {

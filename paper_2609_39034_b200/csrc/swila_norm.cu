@@ -8,7 +8,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include "../../include/swila.h"
+#include "swila_common.cuh"
 
 namespace swila {
 
@@ -121,22 +121,27 @@ template <bool BF16>
 static void launch_rmsnorm(uint4 *o, const float *weight, size_t rows, int Dv, float eps, int sms, cudaStream_t st) {
   const int nvec = Dv / (BF16 ? 8 : 4);
   // 8 warps per block; as many blocks as are resident at once (the kernels stride over the rows), fewer for few rows
-  auto grid_for = [&](auto kern, size_t rows_per_warp) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+  auto grid_for = [&](auto kern, std::atomic<int> &known, size_t rows_per_warp) {
+    int per_sm = known.load(std::memory_order_relaxed);  // (the same on every device: the library is built for one architecture)
+    if (!per_sm) {
+      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1) per_sm = 1;
+      known.store(per_sm, std::memory_order_relaxed);
+    }
     const size_t want = (rows + 8 * rows_per_warp - 1) / (8 * rows_per_warp), cap = (size_t)sms * per_sm;
     return (unsigned)(want < cap ? want : cap);
   };
 #define SWILA_NORM_CASE(LPR)                                                                                   \
   if (nvec <= LPR) {                                                                                           \
+    static std::atomic<int> known;                                                                             \
     auto kern = rmsnorm_rows_kernel<BF16, LPR>;                                                                \
-    kern<<<grid_for(kern, 4 * 32 / LPR), 256, 0, st>>>(o, weight, rows, Dv, eps);                               \
+    kern<<<grid_for(kern, known, 4 * 32 / LPR), 256, 0, st>>>(o, weight, rows, Dv, eps);                               \
     return;                                                                                                    \
   }
   SWILA_NORM_CASE(2) SWILA_NORM_CASE(4) SWILA_NORM_CASE(8) SWILA_NORM_CASE(16) SWILA_NORM_CASE(32)
 #undef SWILA_NORM_CASE
+  static std::atomic<int> known;
   auto kern = rmsnorm_kernel<BF16>;
-  kern<<<grid_for(kern, 1), 256, 0, st>>>(o, weight, rows, Dv, eps);
+  kern<<<grid_for(kern, known, 1), 256, 0, st>>>(o, weight, rows, Dv, eps);
 }
 
 }  // namespace swila
@@ -148,10 +153,8 @@ extern "C" int swila_output_norm(const swila_shape_t *s, void *o, const float *w
   if (reinterpret_cast<uintptr_t>(o) & 15u) return SWILA_ERR_ALIGN;
   const size_t rows = (size_t)s->B * s->H * (size_t)s->T;
   if (rows == 0) return SWILA_OK;
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    return SWILA_ERR_CUDA;
+  const int sms = swila::sm_count();
+  if (!sms) return SWILA_ERR_CUDA;
   if (s->io_dtype == SWILA_IO_BF16)
     swila::launch_rmsnorm<true>((uint4 *)o, weight, rows, s->Dv, eps, sms, (cudaStream_t)stream);
   else

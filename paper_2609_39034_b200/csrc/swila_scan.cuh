@@ -293,6 +293,8 @@ __global__ void __launch_bounds__(C::NT, C::MIN_BLOCKS) swila_scan_kernel(const 
   constexpr int J = C::J, DK = C::DK, NT = C::NT, TB = C::TB, GATE = C::GATE;
   (void)J; (void)DK; (void)NT; (void)TB; (void)GATE;
   constexpr int L = C::L, G = C::G, COLS = C::COLS, S = C::S;
+  launch_next();
+  launch_wait();
   if (p.guard && p.guard_runs_scan && *p.guard == 0u) return;  // the chunked kernel took this call
   extern __shared__ __align__(16) unsigned char smem[];
   float *cooked = reinterpret_cast<float *>(smem + C::OFF_COOKED);
@@ -549,13 +551,27 @@ int launch_scan(const LaunchArgs &a) {
   (void)J; (void)DK; (void)NT; (void)TB; (void)GATE;
   const bool aux = a.p.r_debug || a.p.r_sum || a.p.r_ent || a.p.rho_sum || a.p.rho_ent;
   auto kern = aux ? swila_scan_kernel<C, POST, true> : swila_scan_kernel<C, POST, false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_BYTES);
+  static std::atomic<uint64_t> granted[2];
+  cudaError_t e = allow_smem((const void *)kern, C::SMEM_BYTES, granted[aux]);
   if (e != cudaSuccess) return (int)e;
   const long long nslice = (a.p.Dv + C::COLS - 1) / C::COLS;
   const long long grid = nslice * a.p.B * a.p.H;
   if (grid <= 0 || grid > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
-  kern<<<(unsigned)grid, NT, C::SMEM_BYTES, a.stream>>>(a.p);
-  return (int)cudaGetLastError();
+  // Set up while the launch before it in the stream still runs (a decode step of a small model is as short as its own
+  // launch latency); the kernel starts with launch_wait.
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(NT);
+  cfg.dynamicSmemBytes = C::SMEM_BYTES;
+  cfg.stream = a.stream;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  e = cudaLaunchKernelEx(&cfg, kern, a.p);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return (int)e;
 }
 
 }  // namespace swila

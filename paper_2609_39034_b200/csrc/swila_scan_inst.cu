@@ -29,6 +29,16 @@ int pick(const LaunchArgs &a) {
       if constexpr (GATE == 0 && DK == 128 && J >= 4) return launch_scan<ScanCfg<IO, J, DK, 128, TB, GATE, 16>, POST>(a);
       return -1000;
     }
+    // Few heads: with 128 state values per lane their blocks would not fill the SMs and a warp would spend most of a token in
+    // its own FMAs.  8 key dimensions per lane spread the state over 4 (J = 4) or 2 times as many warps.  The rule looks at
+    // the whole problem and not at T: a prefill and the decode steps that continue it take the same split, hence the same bits.
+    if constexpr ((J == 4 || J == 8) && GATE <= 1) {
+      constexpr int WIDE = ScanCfg<IO, J, DK, 128, TB, GATE>::COLS;
+      if (a.algo != SWILA_ALGO_SCAN_WIDE && a.heads * ((a.p.Dv + WIDE - 1) / WIDE) < sm_count()) {
+        if (a.p.T == 1) return launch_scan<ScanCfg<IO, J, DK, DK, 1, GATE, 8>, POST>(a);
+        return launch_scan<ScanCfg<IO, J, DK, DK, TB, GATE, 8>, POST>(a);
+      }
+    }
     // a decode step stages and prepares one token: blocks of one token (same arithmetic per token, so the bits
     // of a prefill and of the decode steps that continue it still agree)
     if (a.p.T == 1) return launch_scan<ScanCfg<IO, J, DK, 128, 1, GATE>, POST>(a);

@@ -1,0 +1,196 @@
+// Argument marshalling of the calls a program makes once per token or per layer: torch tensors to the C ABI of
+// include/swila.h.  None of the recurrence is here.  What bounds it: a decode step of a small model is a few
+// microseconds on the GPU, and building the argument structs with ctypes took ten on the host.
+#define PY_SSIZE_T_CLEAN
+#include <Python.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "../../include/swila.h"
+
+namespace {
+
+enum Name { N_B, N_H, N_T, N_DK, N_DV, N_J, N_IO, N_FLAGS, N_GRAN, N_Q, N_K, N_V, N_BETA, N_PIK, N_PIQ, N_GK, N_GQ, N_ALPHA, N_W, N_R, N_RHO,
+            N_RSUM, N_RENT, N_QSUM, N_QENT, N_STREAM, N_BF16, N_COUNT };
+const char *const kText[N_COUNT] = {"B", "H", "T", "Dk", "Dv", "J", "io_dtype", "flags", "gate_granularity", "q", "k", "v", "beta_logit",
+                                    "pik_logit", "piq_logit", "gk_logit", "gq_logit", "alpha", "W", "r_prev", "rho_prev", "r_sum", "r_ent",
+                                    "rho_sum", "rho_ent", "cuda_stream", "bf16"};
+PyObject *g_name[N_COUNT];
+
+bool whole(PyObject *obj, int32_t *out) {
+  const long v = PyLong_AsLong(obj);
+  if (v == -1 && PyErr_Occurred()) return false;
+  *out = (int32_t)v;
+  return true;
+}
+bool attr(PyObject *w, Name n, int32_t *out) {
+  PyObject *o = PyObject_GetAttr(w, g_name[n]);
+  if (!o) return false;
+  const bool ok = whole(o, out);
+  Py_DECREF(o);
+  return ok;
+}
+
+// The workload's shape; T is set by the caller.
+bool shape_of(PyObject *w, PyObject *algo, swila_shape_t *s) {
+  if (!attr(w, N_B, &s->B) || !attr(w, N_H, &s->H) || !attr(w, N_DK, &s->Dk) || !attr(w, N_DV, &s->Dv) || !attr(w, N_J, &s->J) ||
+      !attr(w, N_FLAGS, &s->flags) || !attr(w, N_GRAN, &s->gate_granularity) || !whole(algo, &s->algo))
+    return false;
+  PyObject *io = PyObject_GetAttr(w, g_name[N_IO]);
+  if (!io) return false;
+  const int eq = io == g_name[N_BF16] ? 1 : PyObject_RichCompareBool(io, g_name[N_BF16], Py_EQ);
+  Py_DECREF(io);
+  if (eq < 0) return false;
+  s->io_dtype = eq ? SWILA_IO_BF16 : SWILA_IO_FP32;
+  return true;
+}
+
+// A new reference to map[name]; null without an error set when it is missing and not required.
+PyObject *item(PyObject *map, Name n, bool required) {
+  if (PyDict_Check(map)) {
+    PyObject *o = PyDict_GetItemWithError(map, g_name[n]);
+    if (o) return Py_NewRef(o);
+    if (!PyErr_Occurred() && required) PyErr_SetObject(PyExc_KeyError, g_name[n]);
+    return nullptr;
+  }
+  PyObject *o = PyObject_GetItem(map, g_name[n]);
+  if (!o && !required && PyErr_ExceptionMatches(PyExc_KeyError)) PyErr_Clear();
+  return o;
+}
+
+// Device pointer of a tensor (null for None); `layout`: it must be contiguous and on the device.
+bool pointer(PyObject *o, bool layout, void **out) {
+  *out = nullptr;
+  if (!o || o == Py_None) return true;
+  if (!THPVariable_Check(o)) {
+    PyErr_SetString(PyExc_TypeError, "a tensor or None is expected");
+    return false;
+  }
+  const at::Tensor &t = THPVariable_Unpack(o);
+  if (layout && !(t.is_contiguous() && t.is_cuda())) {
+    PyErr_SetString(PyExc_AssertionError, "contiguous tensors on the side the entry point expects");
+    return false;
+  }
+  *out = t.data_ptr();
+  return true;
+}
+bool pointer_at(PyObject *map, Name n, bool required, bool layout, void **out) {
+  PyObject *o = item(map, n, required);
+  if (!o) {
+    *out = nullptr;
+    return !PyErr_Occurred();
+  }
+  const bool ok = pointer(o, layout, out);
+  Py_DECREF(o);
+  return ok;
+}
+
+bool inputs_of(PyObject *inp, void **q, void **k, void **v, swila_gates_t *g) {
+  return pointer_at(inp, N_BETA, false, true, (void **)&g->beta_logit) && pointer_at(inp, N_PIK, false, true, (void **)&g->pik_logit) &&
+         pointer_at(inp, N_PIQ, false, true, (void **)&g->piq_logit) && pointer_at(inp, N_GK, false, true, (void **)&g->gk_logit) &&
+         pointer_at(inp, N_GQ, false, true, (void **)&g->gq_logit) && pointer_at(inp, N_ALPHA, false, true, (void **)&g->alpha) &&
+         pointer_at(inp, N_Q, true, true, q) && pointer_at(inp, N_K, true, true, k) && pointer_at(inp, N_V, true, true, v);
+}
+
+// *given: whether the program passed a state at all (an empty dict counts as none)
+bool state_of(PyObject *st, swila_state_t *s, bool *given) {
+  *given = false;
+  if (st == Py_None) return true;
+  const int truth = PyObject_IsTrue(st);
+  if (truth <= 0) return truth == 0;
+  *given = true;
+  return pointer_at(st, N_W, true, false, (void **)&s->W) && pointer_at(st, N_R, false, false, (void **)&s->r_prev) &&
+         pointer_at(st, N_RHO, false, false, (void **)&s->rho_prev);
+}
+
+bool stream_of(PyObject *obj, void **out) {
+  if (obj == Py_None) {
+    *out = (void *)c10::cuda::getCurrentCUDAStream().stream();
+    return true;
+  }
+  PyObject *o = PyObject_GetAttr(obj, g_name[N_STREAM]);
+  if (!o) return false;
+  *out = PyLong_AsVoidPtr(o);
+  Py_DECREF(o);
+  return !PyErr_Occurred();
+}
+
+bool argc_is(Py_ssize_t n, Py_ssize_t want) {
+  if (n == want) return true;
+  PyErr_Format(PyExc_TypeError, "%zd arguments expected, %zd given", want, n);
+  return false;
+}
+
+// forward(w, inp, state_in, state_out, o, r_debug, stats, algo, stream, T) -> status
+PyObject *forward(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  if (!argc_is(n, 10)) return nullptr;
+  swila_shape_t s;
+  swila_gates_t g;
+  swila_state_t sin, sout;
+  swila_stats_t st;
+  bool has_in, has_out;
+  void *q, *k, *v, *o, *r, *stream;
+  if (!shape_of(a[0], a[7], &s) || !whole(a[9], &s.T) || !inputs_of(a[1], &q, &k, &v, &g) || !state_of(a[2], &sin, &has_in) ||
+      !state_of(a[3], &sout, &has_out) || !pointer(a[4], true, &o) || !pointer(a[5], true, &r) || !stream_of(a[8], &stream))
+    return nullptr;
+  const bool stats = a[6] != Py_None;
+  if (stats && (!pointer_at(a[6], N_RSUM, false, true, (void **)&st.r_sum) || !pointer_at(a[6], N_RENT, false, true, (void **)&st.r_ent) ||
+                !pointer_at(a[6], N_QSUM, false, true, (void **)&st.rho_sum) || !pointer_at(a[6], N_QENT, false, true, (void **)&st.rho_ent)))
+    return nullptr;
+  int rc;
+  Py_BEGIN_ALLOW_THREADS;
+  if (stats) rc = swila_forward_stats(&s, q, k, v, &g, has_in ? &sin : nullptr, has_out ? &sout : nullptr, o, (float *)r, &st, stream);
+  else rc = swila_forward(&s, q, k, v, &g, has_in ? &sin : nullptr, has_out ? &sout : nullptr, o, (float *)r, stream);
+  Py_END_ALLOW_THREADS;
+  return PyLong_FromLong(rc);
+}
+
+// decode(w, inp, state, o, algo, stream) -> status
+PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  if (!argc_is(n, 6)) return nullptr;
+  swila_shape_t s;
+  swila_gates_t g;
+  swila_state_t st;
+  void *q, *k, *v, *o, *stream;
+  if (!shape_of(a[0], a[4], &s) || !inputs_of(a[1], &q, &k, &v, &g) || !pointer_at(a[2], N_W, true, false, (void **)&st.W) ||
+      !pointer_at(a[2], N_R, false, false, (void **)&st.r_prev) || !pointer_at(a[2], N_RHO, false, false, (void **)&st.rho_prev) ||
+      !pointer(a[3], true, &o) || !stream_of(a[5], &stream))
+    return nullptr;
+  s.T = 1;
+  int rc;
+  Py_BEGIN_ALLOW_THREADS;
+  rc = swila_decode_step(&s, q, k, v, &g, &st, o, stream);
+  Py_END_ALLOW_THREADS;
+  return PyLong_FromLong(rc);
+}
+
+// norm(w, o, weight, eps, stream, T) -> status
+PyObject *norm(PyObject *, PyObject *const *a, Py_ssize_t n) {
+  if (!argc_is(n, 6)) return nullptr;
+  swila_shape_t s;
+  void *o, *weight, *stream;
+  PyObject *zero = PyLong_FromLong(0);
+  const bool ok = shape_of(a[0], zero, &s);
+  Py_DECREF(zero);
+  const double eps = PyFloat_AsDouble(a[3]);
+  if (!ok || PyErr_Occurred() || !whole(a[5], &s.T) || !pointer(a[1], true, &o) || !pointer(a[2], true, &weight) || !stream_of(a[4], &stream)) return nullptr;
+  int rc;
+  Py_BEGIN_ALLOW_THREADS;
+  rc = swila_output_norm(&s, o, (const float *)weight, (float)eps, stream);
+  Py_END_ALLOW_THREADS;
+  return PyLong_FromLong(rc);
+}
+
+PyMethodDef kMethods[] = {{"forward", (PyCFunction)(void (*)(void))forward, METH_FASTCALL, nullptr},
+                          {"decode", (PyCFunction)(void (*)(void))decode, METH_FASTCALL, nullptr},
+                          {"norm", (PyCFunction)(void (*)(void))norm, METH_FASTCALL, nullptr},
+                          {nullptr, nullptr, 0, nullptr}};
+PyModuleDef kModule = {PyModuleDef_HEAD_INIT, "_swila_torch", "Marshalling of torch tensors to the SwiLA C ABI.", -1, kMethods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__swila_torch(void) {
+  for (int i = 0; i < N_COUNT; ++i)
+    if (!(g_name[i] = PyUnicode_InternFromString(kText[i]))) return nullptr;
+  return PyModule_Create(&kModule);
+}
