@@ -51,7 +51,8 @@
 // Instantiations: J = 4, 8 at Dk = 64, 128 and J = 16 at Dk = 64; plain, Temporal (App. B.3: the key-side prior
 // mixes in the row's previous responsibility on the serial chain, the readout weights are a running average the
 // helper warps form with the outputs), and an auxiliary one (plain, J <= 8) that also writes the responsibilities
-// and the sums over time behind the load-balancing loss of Sec. 3.5.
+// and the sums over time behind the load-balancing loss of Sec. 3.5.  At Dk = 64 each also with 16 tokens per chunk and two
+// blocks per SM, for launches with enough tiles (see launch_chunk).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -91,13 +92,16 @@ static __device__ unsigned g_chunk_flags[kChunkFlagSlots][kChunkFlagTiles];
 // "Diag(alpha_tj) W" of App. B.4) or one per component.  A row's state is then a scalar multiple of an undecayed
 // one, w_t = A_t (w_0 + sum_{s<=t} (c_s / A_s) k_s) with A_t the product of the row's decays since the chunk began,
 // so the Gram matrices stay shared by all rows and the decay enters as per-row scalars on the FP32 ALUs.
-template <int J_, int DK_, bool TEMPORAL_ = false, bool GATED_ = false>
+template <int J_, int DK_, bool TEMPORAL_ = false, bool GATED_ = false, int C_ = 32>
 struct ChunkCfg {
   static constexpr int J = J_, DK = DK_;
   static constexpr bool TEMPORAL = TEMPORAL_, GATED = GATED_;
-  static constexpr int C = 32;            // tokens per chunk
-  static constexpr int WIN = 24;          // tokens ahead (incl. its own trip) that a token's pushes reach on the ALUs;
-                                          // the pushes of tokens 0-7 into tokens 24-31 go through the tensor cores
+  static constexpr int C = C_;            // tokens per chunk: 32, or 16 with two blocks per SM (Dk = 64)
+  static constexpr bool FARP = C == 32;   // far pushes
+  static constexpr int BLOCKS = C == 32 ? 1 : 2;  // resident blocks per SM
+  static constexpr int NSLOT = 64 / C;    // chunks side by side in the operand tile
+  static constexpr int WIN = FARP ? 24 : C;  // tokens ahead (incl. its own trip) that a token's pushes reach on the ALUs;
+                                          // with 32 tokens those of tokens 0-7 into tokens 24-31 go through the tensor cores
   static constexpr int GT = 8;            // tokens per trip of the rolled loops (keeps the hot code inside the instruction cache)
   static constexpr int NROW = 128;        // row threads = rows of the tile
   static constexpr int NT = GATED_ ? 320 : 288;  // 4 row warps + 4 helper warps + 1 MMA warp (+ 1 decay warp when Gated)
@@ -109,19 +113,20 @@ struct ChunkCfg {
   // the chunk add to the predictions of its last 16 (only the last 8 are non-zero); CHI / CLO / CL3: the bf16 parts of the
   // chunk's update coefficients, two tokens per column (the third part is an operand of the state update only)
   static constexpr int TM_W = 0, TM_WHI = DK, TM_WLO = DK + DK / 2, TM_PQ = 2 * DK, TM_QD = TM_PQ + 2 * C,
-                       TM_G = TM_QD + 2 * C, TM_FAR = TM_G + 2 * C, TM_CHI = TM_FAR + C / 2, TM_CLO = TM_CHI + C / 2,
+                       TM_G = TM_QD + 2 * C, TM_FAR = TM_G + 2 * C, TM_CHI = TM_FAR + (FARP ? C / 2 : 0), TM_CLO = TM_CHI + C / 2,
                        TM_CL3 = TM_CLO + C / 2, TM_USED = TM_CL3 + C / 2;
-  static constexpr int TM_ALLOC = 512;
+  static constexpr int TM_ALLOC = 512 / BLOCKS;
+  static_assert(C == 32 || (C == 16 && DK == 64), "two blocks per SM: tensor memory holds them at Dk = 64 only");
   static_assert(TM_USED <= TM_ALLOC, "tensor memory budget");
   static_assert(J == 4 || J == 8 || (J == 16 && DK == 64),
                 "J = 4, 8: outputs by in-group transposition; J = 16: by shuffle sums, and only Dk = 64 fits shared memory");
   // K/Q operand tile (bf16, K-major, 128-byte swizzle): per half of 64 key dims, 128 rows of 128 bytes, rows
-  // [K_even ; Q_even ; K_odd ; Q_odd]: the chunks of both parities side by side, so that one 128-row A operand
-  // covers the keys of two consecutive chunks.  Key dim d of row r sits at
+  // [K ; Q] of NSLOT consecutive chunks (chunk m in slot m % NSLOT) side by side: one 128-row A operand, of which a Gram batch
+  // uses the rows of its own chunk; they are the tensor-memory lanes of two helper warps (32 tokens) or of one (16).  Key dim d of row r sits at
   //   (d / 64) * TILE_HALF + r * 128 + (((d / 8) % 8) ^ (r % 8)) * 16 + (d % 8) * 2,
   // which is what a tensor copy with the 128-byte swizzle mode writes: k and q go straight from global memory
   // into the tile, 4 KB per copy.
-  static constexpr int TILE_HALF = 4 * C * 128;
+  static constexpr int TILE_HALF = NSLOT * 2 * C * 128;
   static constexpr int TILE_BYTES = (DK / 64) * TILE_HALF;
   // A second copy of a chunk's keys for the update MMA, which reads them MN-major (tokens = K index) after the
   // chunk, when the tile rows are already being refilled: 3-deep ring of [DK/64][C rows][128 bytes], same swizzle.
@@ -173,7 +178,7 @@ struct ChunkCfg {
   static constexpr int FAR_LBO = (C / 2) * 16;     // far-push operand: rows = tokens 16..31, K index = tokens 0..15
   static constexpr int FAR_TILE = 2 * FAR_LBO;
   static constexpr int OFF_FAR = OFF_OST + 2 * C * COLS * ES;  // 2 x { hi, lo }
-  static constexpr int OFF_P0 = OFF_FAR + 2 * 2 * FAR_TILE;  // [C/4][NROW] float4: a chunk's P0 rows, kept for the rare redo
+  static constexpr int OFF_P0 = OFF_FAR + (FARP ? 2 * 2 * FAR_TILE : 0);  // [C/4][NROW] float4: a chunk's P0 rows, kept for the rare redo
   static constexpr int OFF_RP = OFF_P0 + C * NROW * 4;  // Temporal: [NROW] fp32, a piece's initial r_prev, helpers -> row warps
   static constexpr int OFF_OS = OFF_RP + (TEMPORAL ? NROW * 4 : 0);  // J = 16: [C][COLS][J] fp32, a chunk's readouts regrouped by output
   // Gated: 2 x [C + 1][NROW] fp32, the running products of a chunk's decays per row: entry t + 1 holds A_t, entry 0
@@ -190,7 +195,7 @@ struct ChunkCfg {
   static_assert(RAW_BYTES % 128 == 0 && RPQ_BYTES % 128 == 0 && R_B % 128 == 0 && R_PK % 128 == 0 && OFF_RAW % 128 == 0 &&
                     OFF_RPQ % 128 == 0 && OFF_TILE % 1024 == 0 && OFF_KU % 1024 == 0 && KU_BYTES % 1024 == 0 && DK % 64 == 0 && (COLS * ES) % 16 == 0 && (GROW * ES) % 16 == 0,
                 "destinations of the tensor copies are 128-byte aligned, their rows multiples of 16 bytes");
-  static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
+  static_assert(BLOCKS * (SMEM_BYTES + 1024) <= 228 * 1024, "shared memory budget (1 KB per block is the system's)");
 };
 
 // barrier slots.  Committed by the MMA thread: E (state x [K;Q] of a chunk complete), G (Gram batch), U (update of W),
@@ -240,7 +245,7 @@ __device__ __forceinline__ void chunk_stage(const ChunkMaps &maps, unsigned char
   constexpr int DK = Cf::DK, C = Cf::C;
   fence_async_smem();  // the buffers were last read through ordinary loads
   mbar_arrive_expect_tx(bar, Cf::STAGE_TX_BYTES + (ku_mirror ? C * DK * Cf::ES : 0));
-  unsigned char *trow = tile + (m & 1) * 2 * C * 128;  // this chunk's 2C rows of the operand tile
+  unsigned char *trow = tile + (m % Cf::NSLOT) * 2 * C * 128;  // this chunk's 2C rows of the operand tile
 #pragma unroll
   for (int hf = 0; hf < DK / 64; ++hf) {
     tma_load_3d(trow + hf * Cf::TILE_HALF, &maps.k, hf * 64, tok, bh, bar);
@@ -262,7 +267,7 @@ __device__ __forceinline__ void chunk_stage(const ChunkMaps &maps, unsigned char
 // over time of the mixture weights (Sec. 3.5) to p.r_sum, p.r_ent, p.rho_sum, p.rho_ent; each pointer is tested at
 // run time there, none of it is in the plain instantiation.
 template <class Cf, bool RDEBUG>
-__global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_constant__ ScanParams p,
+__global__ void __launch_bounds__(Cf::NT, Cf::BLOCKS) swila_chunk_kernel(const __grid_constant__ ScanParams p,
                                                                      const __grid_constant__ ChunkSched sched,
                                                                      const __grid_constant__ ChunkMaps maps) {
   using namespace umma;
@@ -348,7 +353,7 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
     mbar_init(&bars[B_KQ0], 1);  // the thread that issues the tensor copies
     mbar_init(&bars[B_KQ1], 1);
     mbar_init(&bars[B_WP], 128);
-    mbar_init(&bars[B_GS], 64);
+    mbar_init(&bars[B_GS], Cf::FARP ? 64 : 32);
     mbar_init(&bars[B_C], 128);
     mbar_init(&bars[B_PQF], 128);
     mbar_init(&bars[B_BE], 128);
@@ -637,8 +642,8 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
           if constexpr (Cf::GATED) P(t) = -pred0[t];
           else P(t) = __bfloat162float(rv[t * COLS + dl]) - pred0[t];
         }
-        [[maybe_unused]] float p0late[C - Cf::WIN];
-        if constexpr (!EXACT) {
+        [[maybe_unused]] float p0late[8];
+        if constexpr (!EXACT && Cf::FARP) {
 #pragma unroll
           for (int t = 0; t < C - Cf::WIN; ++t) {
             if constexpr (Cf::GATED) p0late[t] = -pred0[Cf::WIN + t];
@@ -648,7 +653,7 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
         float c_prev = 0.f;
 #pragma unroll 1
         for (int tg = 0; tg < C; tg += GT) {
-          if constexpr (!EXACT) {
+          if constexpr (!EXACT && Cf::FARP) {
             if (tg == Cf::WIN) {  // far pushes of tokens 0-6 into tokens 24-31
               if (!mbar_wait(&bars[B_FAR], n & 1)) failed = true;
               tc_fence_after_sync();
@@ -756,7 +761,7 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
             tmem_st4(tb + Cf::TM_CLO + tg / 2, lo);
             tmem_st4(tb + Cf::TM_CL3 + tg / 2, l3);
           }
-          if constexpr (!EXACT) {
+          if constexpr (!EXACT && Cf::FARP) {
             // the coefficients of tokens 0-15 are in place: the far pushes (of tokens 0-7, needed at token 24) and the
             // first half of the cross-chunk term may be issued
             if (tg == GT) {
@@ -769,7 +774,7 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
           for (int i = 0; i + GT < WINS; i += 2) pred2[i / 2] = pred2[(i + GT) / 2];
 #pragma unroll
           for (int i = 0; i < GT; ++i) {  // the slots that enter the window: tokens 24-31 after the first trip, dead later
-            if constexpr (EXACT) {
+            if constexpr (EXACT || !Cf::FARP) {
               P(WINS - GT + i) = 0.f;
             } else {
               P(WINS - GT + i) = p0late[i];
@@ -949,7 +954,9 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
     //   query rows (lane t):  Q_m K_m^T, causally masked (s <= t), as the hi / lo operand of the readout MMA;
     //   both:                 [K_m;Q_m] K_{m-1}^T as the hi / lo operand of the cross-chunk MMA.
     auto spill_gram = [&](int m) {
-      const bool qrows = (warp & 1) != 0;
+      // 32 tokens: a warp of keys and a warp of queries; 16 tokens: both halves of one warp
+      const bool qrows = Cf::FARP ? (warp & 1) != 0 : lane >= C;
+      const int row = Cf::FARP ? lane : lane % C;  // token
       float a[C];
 #pragma unroll
       for (int cc = 0; cc < C / 16; ++cc) tmem_ld16(tb + Cf::TM_G + C + cc * 16, reinterpret_cast<float(&)[16]>(a[cc * 16]));
@@ -958,39 +965,43 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
         float *Gkk = G_all + (m & 1) * C * C;
 #pragma unroll
         for (int i = 0; i < C / 4; ++i)
-          *reinterpret_cast<float4 *>(Gkk + lane * C + i * 4) = make_float4(-a[4 * i], -a[4 * i + 1], -a[4 * i + 2], -a[4 * i + 3]);
+          *reinterpret_cast<float4 *>(Gkk + row * C + i * 4) = make_float4(-a[4 * i], -a[4 * i + 1], -a[4 * i + 2], -a[4 * i + 3]);
         // far-push operand: row = token u = lane (16..31), K index = tokens 0..7 (K K^T is symmetric, so this lane's
         // row holds k_s.k_u).  Through the tensor cores go the pushes of tokens s = 0..6 into tokens u >= WIN: the row
         // warps push token s into tokens s+1 .. 23 while they are in the first trip, and token 7, whose deferred push
         // runs in the second trip, reaches token 31 there.  Everything else in the operand is zero.
-        if (lane >= C / 2) {
-          uint32_t hi[4], lo[4];
+        if constexpr (Cf::FARP) {
+          if (lane >= C / 2) {
+            uint32_t hi[4], lo[4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const bool use = lane >= Cf::WIN;
-            bf16_split2(use ? a[2 * i] : 0.f, (use && 2 * i + 1 < Cf::GT - 1) ? a[2 * i + 1] : 0.f, hi[i], lo[i]);
+            for (int i = 0; i < 4; ++i) {
+              const bool use = lane >= Cf::WIN;
+              bf16_split2(use ? a[2 * i] : 0.f, (use && 2 * i + 1 < Cf::GT - 1) ? a[2 * i + 1] : 0.f, hi[i], lo[i]);
+            }
+            unsigned char *ft = smem + Cf::OFF_FAR + (m & 1) * 2 * Cf::FAR_TILE;
+            *reinterpret_cast<uint4 *>(ft + (lane - C / 2) * 16) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4 *>(ft + Cf::FAR_TILE + (lane - C / 2) * 16) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
           }
-          unsigned char *ft = smem + Cf::OFF_FAR + (m & 1) * 2 * Cf::FAR_TILE;
-          *reinterpret_cast<uint4 *>(ft + (lane - C / 2) * 16) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-          *reinterpret_cast<uint4 *>(ft + Cf::FAR_TILE + (lane - C / 2) * 16) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
       } else {
 #pragma unroll
-        for (int s = 0; s < C; ++s) a[s] = (s <= lane) ? a[s] : 0.f;
+        for (int s = 0; s < C; ++s) a[s] = (s <= row) ? a[s] : 0.f;
         unsigned char *bq = BQ_all + (m & 1) * 2 * Cf::BQ_TILE;
-        store_parts(a, bq, bq + Cf::BQ_TILE, Cf::BQ_LBO, lane);
+        store_parts(a, bq, bq + Cf::BQ_TILE, Cf::BQ_LBO, row);
       }
       if (m > 0) {
+        __syncwarp();
 #pragma unroll
         for (int cc = 0; cc < C / 16; ++cc)
           tmem_ld16(tb + Cf::TM_G + cc * 16, reinterpret_cast<float(&)[16]>(a[cc * 16]));
         tmem_ld_wait();
-        store_parts(a, GX_all, GX_all + Cf::GX_TILE, Cf::GX_LBO, (qrows ? C : 0) + lane);
+        store_parts(a, GX_all, GX_all + Cf::GX_TILE, Cf::GX_LBO, (qrows ? C : 0) + row);
       }
       tc_fence_before_sync();
       fence_async_smem();
     };
-    const bool spill_mine[2] = {warp < 6, warp >= 6};  // which parity of chunks this warp's lanes hold
+    // whether this warp's lanes hold the rows of chunk m
+    auto spill_mine = [&](int m) { return Cf::FARP ? ((warp - 4) >> 1) == (m & 1) : warp - 4 == m % Cf::NSLOT; };
 
     // ---- prologue: stage chunks 0 and 1, state row -> tensor memory, operands of chunk 0 ----
     // stage chunk m of this piece (one thread; the buffers it overwrites were last read through ordinary loads,
@@ -1071,11 +1082,12 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
     }
     // the far-push MMA spans 16 tokens of coefficients and of its operand, of which only the first 8 count: the
     // operand's other half stays zero, and the coefficient columns must at least be finite from the start
-    for (int e = h; e < 4 * (C / 2); e += 128)
+    for (int e = h; Cf::FARP && e < 4 * (C / 2); e += 128)
       *reinterpret_cast<uint4 *>(smem + Cf::OFF_FAR + (e / (C / 2)) * Cf::FAR_TILE + Cf::FAR_LBO + (e % (C / 2)) * 16) = make_uint4(0, 0, 0, 0);
-    if (nchunks == 1) {  // the odd half of the operand tile is read (as don't-care rows) by the Gram batch: make it finite
-      for (int e = h; e < (DK / 64) * 2 * C * 8; e += 128)
-        *reinterpret_cast<uint4 *>(tile + (e / (2 * C * 8)) * Cf::TILE_HALF + 2 * C * 128 + (e % (2 * C * 8)) * 16) = make_uint4(0, 0, 0, 0);
+    if (nchunks < Cf::NSLOT) {  // the other slots of the operand tile are read (as don't-care rows) by the Gram batch: make them finite
+      const int rows = (Cf::NSLOT - nchunks) * 2 * C;
+      for (int e = h; e < (DK / 64) * rows * 8; e += 128)
+        *reinterpret_cast<uint4 *>(tile + (e / (rows * 8)) * Cf::TILE_HALF + nchunks * 2 * C * 128 + (e % (rows * 8)) * 16) = make_uint4(0, 0, 0, 0);
     }
     if (!staged(0)) failed = true;
     {
@@ -1088,7 +1100,7 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
     }
     if constexpr (Cf::TEMPORAL) cook_pk(smem + Cf::OFF_RAW);
     mbar_arrive(&bars[B_BE]);
-    if (spill_mine[0]) {
+    if (spill_mine(0)) {
       if (!mbar_wait(&bars[B_G], 0)) failed = true;
       tc_fence_after_sync();
       if (!failed) spill_gram(0);
@@ -1127,7 +1139,7 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
         cook_be(smem + Cf::OFF_RAW + ((n + 1) & 1) * Cf::RAW_BYTES, min(C, Tseg - (n + 1) * C), As1);
         if constexpr (Cf::TEMPORAL) cook_pk(smem + Cf::OFF_RAW + ((n + 1) & 1) * Cf::RAW_BYTES);
         mbar_arrive(&bars[B_BE]);
-        if (spill_mine[(n + 1) & 1]) {
+        if (spill_mine(n + 1)) {
           if (!mbar_wait(&bars[B_G], (n + 1) & 1)) failed = true;
           tc_fence_after_sync();
           if (!failed) spill_gram(n + 1);
@@ -1269,10 +1281,10 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
     auto w_times_kq = [&](int m) {
 #pragma unroll 1
       for (int ks = 0; ks < DK / 16; ++ks)
-        mma_bf16_ts(tb0 + Cf::TM_PQ, tb0 + Cf::TM_WHI + ks * 8, tile_desc((m & 1) * 2 * C, ks), idE, ks > 0);
+        mma_bf16_ts(tb0 + Cf::TM_PQ, tb0 + Cf::TM_WHI + ks * 8, tile_desc((m % Cf::NSLOT) * 2 * C, ks), idE, ks > 0);
 #pragma unroll 1
       for (int ks = 0; ks < DK / 16; ++ks)
-        mma_bf16_ts(tb0 + Cf::TM_PQ, tb0 + Cf::TM_WLO + ks * 8, tile_desc((m & 1) * 2 * C, ks), idE, true);
+        mma_bf16_ts(tb0 + Cf::TM_PQ, tb0 + Cf::TM_WLO + ks * 8, tile_desc((m % Cf::NSLOT) * 2 * C, ks), idE, true);
     };
     // + Cmat (K_prev [K;Q]^T): the update of the chunk that just finished, seen by the next chunk's products
     // (16 tokens of the chunk per call)
@@ -1314,7 +1326,7 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
         tc_fence_after_sync();
         gram(n + 1);
       }
-      {
+      if constexpr (Cf::FARP) {
         // far pushes of chunk n: what its first 8 tokens add to the predictions of its last 8, needed when the row
         // warps reach token 24.  A = the coefficient columns of tokens 0..15 (8..15 are stale but finite and meet
         // zero rows of the operand), B = rows 16..31 of K K^T against tokens 0..7.
@@ -1334,18 +1346,18 @@ __global__ void __launch_bounds__(Cf::NT, 1) swila_chunk_kernel(const __grid_con
         // chunk still runs
         if (!mbar_wait(&bars[B_GS], (n + 1) & 1)) { failed = true; break; }
         tc_fence_after_sync();
-        cross(0);
+        if constexpr (Cf::FARP) cross(0);
       }
       if (!mbar_wait(&bars[B_C], n & 1)) { failed = true; break; }
       tc_fence_after_sync();
-      const bool redone = *redo_s != 0;  // ordered by the barrier: set before the row warps arrived
+      const bool redone = Cf::FARP && *redo_s != 0;  // ordered by the barrier: set before the row warps arrived
       if (redone) *redo_s = 0;
       if (more) {
         if (redone) {  // rare: a row warp replaced the coefficients that the first half was formed from
           w_times_kq(n + 1);
           cross(0);
         }
-        cross(1);  // -> E(n+1): the only tensor work left between two chunks of the row warps
+        cross(C / 16 - 1);  // -> E(n+1): the only tensor work left between two chunks of the row warps
         mma_commit(&bars[B_E]);
       }
       if constexpr (Cf::GATED) {
@@ -1421,9 +1433,9 @@ inline unsigned chunk_next_epoch() {
   return e;
 }
 
-template <int J, int DK, bool TEMPORAL = false, bool GATED = false>
-int launch_chunk(const LaunchArgs &a) {
-  using Cf = ChunkCfg<J, DK, TEMPORAL, GATED>;
+template <int J, int DK, bool TEMPORAL, bool GATED, int C>
+int launch_chunk_c(const LaunchArgs &a) {
+  using Cf = ChunkCfg<J, DK, TEMPORAL, GATED, C>;
   const bool aux = a.p.r_debug || a.p.r_sum || a.p.r_ent || a.p.rho_sum || a.p.rho_ent;
   if (J > 8 && aux) return -1000;     // likewise for J = 16
   if (GATED && aux) return -1000;     // and for the Gated variant
@@ -1447,7 +1459,7 @@ int launch_chunk(const LaunchArgs &a) {
   // tiles, so that the last wave is not half empty (chunk_plan).  The state of a split tile travels through the
   // state output, hence only when that is given; blocks of such a launch wait for each other, hence the
   // cooperative launch (all blocks resident or no launch at all).
-  const ChunkPlan pl = chunk_plan((long long)a.p.B * a.p.H, nslice, nch, sm_count(),
+  const ChunkPlan pl = chunk_plan((long long)a.p.B * a.p.H, nslice, nch, sm_count() * Cf::BLOCKS,
                                    a.p.W_out != nullptr && (!TEMPORAL || (a.p.r_out && a.p.rho_out)), kChunkFlagTiles);
   if (pl.split) {
     static std::atomic<unsigned *> flags_of[kMaxDevices];
@@ -1469,6 +1481,19 @@ int launch_chunk(const LaunchArgs &a) {
   }
   kern<<<(unsigned)ntiles, Cf::NT, Cf::SMEM_BYTES, a.stream>>>(prm, sc, maps);
   return (int)cudaGetLastError();
+}
+
+// Tokens per chunk.  At Dk = 64 two blocks with chunks of 16 tokens fit an SM (tensor memory 2 x 256 columns) and fill each other's
+// waits; one block alone is faster with chunks of 32, whose cross-chunk steps come half as often.  Measured at 2048 tokens, J = 4,
+// per wave of 148 (C = 32) or 296 (C = 16) tiles: plain 266 and 452 us, with the statistics 406 and 587, row gates 361 and 555: the two
+// meet at 1.6 to 1.7 tiles per SM.  Temporal gains nothing from it (1,288 against 1,258 us at 16 x 8 heads, 4096 tokens).
+template <int J, int DK, bool TEMPORAL = false, bool GATED = false>
+int launch_chunk(const LaunchArgs &a) {
+  if constexpr (DK == 64 && !TEMPORAL) {
+    const long long cols = 128 / J, tiles = a.heads * ((a.p.Dv + cols - 1) / cols);
+    if (10 * tiles >= 17 * sm_count()) return launch_chunk_c<J, DK, TEMPORAL, GATED, 16>(a);
+  }
+  return launch_chunk_c<J, DK, TEMPORAL, GATED, 32>(a);
 }
 
 }  // namespace swila
