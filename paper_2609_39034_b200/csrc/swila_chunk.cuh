@@ -650,11 +650,30 @@ __global__ void __launch_bounds__(Cf::NT, Cf::BLOCKS) swila_chunk_kernel(const _
             else p0late[t] = __bfloat162float(rv[(Cf::WIN + t) * COLS + dl]) - pred0[Cf::WIN + t];
           }
         }
-        float c_prev = 0.f;
+        // Gates one token ahead.  With two blocks per SM, where registers are short, these loads and the Gram rows' are pinned
+        // where they are written, under the latency of the shuffles (left to itself the compiler then puts them in front of
+        // their uses: 2,100 cycles per trip against 1,760); with one block they are the compiler's to place (pinned: 1 to 3 % slower).
+        constexpr bool PIN = Cf::BLOCKS == 2;
+        float be_next, pk_next;
+        [[maybe_unused]] float gk_next = 0.f, v_next = 0.f, as_next = 0.f;
+        auto fetch = [&](int t) {
+          be_next = lds_f32<PIN>(bes + t * NROW + r);
+          if constexpr (Cf::TEMPORAL) {
+            pk_next = lds_f32<PIN>(pks + t * NROW + r);
+            gk_next = sigmoid_approx(lds_bf16<PIN>(rgk + t * COLS + dl));
+          } else {
+            pk_next = lds_bf16<PIN>(rpk + (t * J + j) * Cf::GROW + dl) * kLog2e;
+          }
+          if constexpr (Cf::GATED) {
+            as_next = lds_f32<PIN>(As + (t + a_off) * NROW + a_slot);
+            v_next = lds_bf16<PIN>(rv + t * COLS + dl);
+          }
+        };
+        fetch(0);
 #pragma unroll 1
         for (int tg = 0; tg < C; tg += GT) {
           if constexpr (!EXACT && Cf::FARP) {
-            if (tg == Cf::WIN) {  // far pushes of tokens 0-6 into tokens 24-31
+            if (tg == Cf::WIN) {  // far pushes of tokens 0-7 into tokens 24-31
               if (!mbar_wait(&bars[B_FAR], n & 1)) failed = true;
               tc_fence_after_sync();
               float far[8];
@@ -665,32 +684,49 @@ __global__ void __launch_bounds__(Cf::NT, Cf::BLOCKS) swila_chunk_kernel(const _
             }
           }
           float cs[GT];
+          float gr[WINS];  // minus the products of one token's key with those of the window's slots
+          auto push = [&](int i) {  // token tg + i into the slots from i + 2 on
+            if (i & 1) P(i + 2) = fmaf(cs[i], gr[i + 2], P(i + 2));
+#pragma unroll
+            for (int u = (i + 3) / 2; u < WINS / 2; ++u) pred2[u] = __ffma2_rn(make_float2(cs[i], cs[i]), make_float2(gr[2 * u], gr[2 * u + 1]), pred2[u]);
+          };
 #pragma unroll
           for (int i = 0; i < GT; ++i) {
             const int t = tg + i;
-            const float be = bes[t * NROW + r];
+            const float be = be_next;
             // serial chain: prediction error -> responsibilities (Eq. 3.4) -> update coefficient (Eq. 3.3)
             // Gated: delta = v - A (w_0.k + sum_s (c_s / A_s) k_s.k), A = the row's decay product up to this token
             // (pre-decay, Eq. 3.8) or up to the previous one (post-decay, Eq. 3.7); beta arrives divided by A_t, so
             // that the coefficient below is already c_t / A_t
             float delta;
-            if constexpr (Cf::GATED) delta = fmaf(As[(t + a_off) * NROW + a_slot], P(i), __bfloat162float(rv[t * COLS + dl]));
+            if constexpr (Cf::GATED) delta = fmaf(as_next, P(i), v_next);
             else delta = P(i);
             float a;
             if constexpr (Cf::TEMPORAL) {
               // key-side prior (1 - g) r_{t-1} + g pi^k with g = sigmoid(gk logit) (App. B.3): a convex combination of
               // two distributions over j, so it needs no further normalisation
-              const float gk = sigmoid_approx(__bfloat162float(rgk[t * COLS + dl]));
-              const float prior = fmaf(gk, pks[t * NROW + r] - rp, rp);
+              const float prior = fmaf(gk_next, pk_next - rp, rp);
               a = fmaf(-kHalfLog2e * delta, delta, lg2_approx(prior));
             } else {
-              a = fmaf(-kHalfLog2e * delta, delta, __bfloat162float(rpk[(t * J + j) * Cf::GROW + dl]) * kLog2e);
+              a = fmaf(-kHalfLog2e * delta, delta, pk_next);
             }
+            // Under the latency of the shuffles: the previous token's pushes (only its push into this token stood on the serial
+            // chain), this token's Gram row, the next token's gates (past the chunk's last token: inside the stage, unused)
+            auto shadow = [&]() {
+              if (i > 0) push(i - 1);
+#pragma unroll
+              for (int q = (i + 1) / 4; q < WINS / 4; ++q) {
+                const float4 g4 = lds_f32x4<PIN>(Gkk + t * C + tg + 4 * q);
+                gr[4 * q] = g4.x; gr[4 * q + 1] = g4.y; gr[4 * q + 2] = g4.z; gr[4 * q + 3] = g4.w;
+              }
+              fetch(t + 1);
+            };
             float e, sum;
             if constexpr (EXACT) {
               float all[J];
 #pragma unroll
               for (int jj = 0; jj < J; ++jj) all[jj] = __shfl_sync(0xffffffffu, a, jbase + jj);
+              shadow();
               float m = all[0];
 #pragma unroll
               for (int jj = 1; jj < J; ++jj) m = fmaxf(m, all[jj]);
@@ -705,6 +741,7 @@ __global__ void __launch_bounds__(Cf::NT, Cf::BLOCKS) swila_chunk_kernel(const _
                 part[0] = e;
 #pragma unroll
                 for (int jj = 1; jj < J; ++jj) part[jj] = __shfl_sync(0xffffffffu, e, jbase + ((j + jj) & (J - 1)));
+                shadow();
 #pragma unroll
                 for (int w = J / 2; w >= 1; w /= 2) {
 #pragma unroll
@@ -714,21 +751,13 @@ __global__ void __launch_bounds__(Cf::NT, Cf::BLOCKS) swila_chunk_kernel(const _
               } else {  // 15 shuffles per token cost more than the latency of 4 dependent rounds
                 sum = e;
 #pragma unroll
-                for (int off = 1; off < J; off <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, off);
+                for (int off = 1; off < J; off <<= 1) {
+                  const float y = __shfl_xor_sync(0xffffffffu, sum, off);
+                  if (off == 1) shadow();
+                  sum += y;
+                }
               }
               bad = bad || !(sum > 1e-30f && sum < 1e30f);
-            }
-            {  // deferred push of token t-1 into the predictions of tokens t+1 .. (slots i+1 ..)
-              const float4 *gp = reinterpret_cast<const float4 *>(Gkk + max(t - 1, 0) * C + tg);
-#pragma unroll
-              for (int u4 = (i + 1) / 4; u4 < WINS / 4; ++u4) {
-                const float4 g = gp[u4];
-                const float2 cc = make_float2(c_prev, c_prev);
-                if (4 * u4 + 0 > i) pred2[2 * u4] = __ffma2_rn(cc, make_float2(g.x, g.y), pred2[2 * u4]);
-                else if (4 * u4 + 1 > i) pred2[2 * u4].y = fmaf(c_prev, g.y, pred2[2 * u4].y);
-                if (4 * u4 + 2 > i) pred2[2 * u4 + 1] = __ffma2_rn(cc, make_float2(g.z, g.w), pred2[2 * u4 + 1]);
-                else if (4 * u4 + 3 > i) pred2[2 * u4 + 1].y = fmaf(c_prev, g.w, pred2[2 * u4 + 1].y);
-              }
             }
             const float rs = rcp_approx(sum);
             float c = ((be * delta) * e) * rs;  // beta r delta with one multiplication after the reciprocal
@@ -745,9 +774,9 @@ __global__ void __launch_bounds__(Cf::NT, Cf::BLOCKS) swila_chunk_kernel(const _
                 if (rr > 0.f) ch = fmaf(rr, lg2_approx(e) - lg2_approx(sum), ch);
               }
             }
-            P(i + 1) = fmaf(c, Gkk[t * C + t + 1], P(i + 1));  // the push the next token waits for
-            c_prev = c;
+            P(i + 1) = fmaf(c, gr[i + 1], P(i + 1));  // the push the next token waits for
           }
+          push(GT - 1);
           // the coefficient columns are still operands of the previous chunk's update and readout MMAs until
           // those complete (normally long before the first trip ends)
           if (tg == 0 && n > 0) {
@@ -967,16 +996,15 @@ __global__ void __launch_bounds__(Cf::NT, Cf::BLOCKS) swila_chunk_kernel(const _
         for (int i = 0; i < C / 4; ++i)
           *reinterpret_cast<float4 *>(Gkk + row * C + i * 4) = make_float4(-a[4 * i], -a[4 * i + 1], -a[4 * i + 2], -a[4 * i + 3]);
         // far-push operand: row = token u = lane (16..31), K index = tokens 0..7 (K K^T is symmetric, so this lane's
-        // row holds k_s.k_u).  Through the tensor cores go the pushes of tokens s = 0..6 into tokens u >= WIN: the row
-        // warps push token s into tokens s+1 .. 23 while they are in the first trip, and token 7, whose deferred push
-        // runs in the second trip, reaches token 31 there.  Everything else in the operand is zero.
+        // row holds k_s.k_u).  Through the tensor cores go the pushes of tokens s = 0..7 into tokens u >= WIN: the row
+        // warps push them into tokens s+1 .. 23, the reach of the first trip.  Everything else in the operand is zero.
         if constexpr (Cf::FARP) {
           if (lane >= C / 2) {
             uint32_t hi[4], lo[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const bool use = lane >= Cf::WIN;
-              bf16_split2(use ? a[2 * i] : 0.f, (use && 2 * i + 1 < Cf::GT - 1) ? a[2 * i + 1] : 0.f, hi[i], lo[i]);
+              bf16_split2(use ? a[2 * i] : 0.f, use ? a[2 * i + 1] : 0.f, hi[i], lo[i]);
             }
             unsigned char *ft = smem + Cf::OFF_FAR + (m & 1) * 2 * Cf::FAR_TILE;
             *reinterpret_cast<uint4 *>(ft + (lane - C / 2) * 16) = make_uint4(hi[0], hi[1], hi[2], hi[3]);

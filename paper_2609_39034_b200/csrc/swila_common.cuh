@@ -77,6 +77,8 @@ int scan_dispatch(const LaunchArgs &a);
 // Likewise for the blocked scan; err: the device word an expired wait leaves its code in.
 template <int DK, int GATE>
 int block_dispatch(const LaunchArgs &a, int *err, int sms);
+template <int DK, bool BF16>
+int tile_dispatch(const LaunchArgs &a, int *err, int sms);
 
 // ---------------------------------------------------------------------------------------
 constexpr float kLog2e = 1.4426950408889634f;
@@ -123,6 +125,29 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Shared-memory loads; with PIN they stay where they are written, among shuffles, barriers and one another.
+template <bool PIN>
+__device__ __forceinline__ float lds_f32(const float *p) {
+  if constexpr (!PIN) return *p;
+  float x;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"((unsigned)__cvta_generic_to_shared(p)));
+  return x;
+}
+template <bool PIN>
+__device__ __forceinline__ float lds_bf16(const __nv_bfloat16 *p) {
+  if constexpr (!PIN) return __bfloat162float(*p);
+  unsigned short x;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"((unsigned)__cvta_generic_to_shared(p)));
+  return __uint_as_float((uint32_t)x << 16);
+}
+template <bool PIN>
+__device__ __forceinline__ float4 lds_f32x4(const float *p) {
+  if constexpr (!PIN) return *reinterpret_cast<const float4 *>(p);
+  float4 x;
+  asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"((unsigned)__cvta_generic_to_shared(p)));
+  return x;
 }
 
 // Two FP32 FMAs / multiplies on a register pair.  SWILA_SCALAR_FMA selects plain scalar
