@@ -55,8 +55,14 @@ def _units():
         for gate, post in GATE_MODES:
             units.append((f"scan_dk{dk}_g{gate}_p{post}.o", os.path.join(CSRC, "swila_scan_inst.cu"),
                           [f"-DSWILA_DK={dk}", f"-DSWILA_GATE={gate}", f"-DSWILA_POST={post}"]))
+        for gate in ((0, 1, 2) if dk == 16 else (1, 2)):
+            units.append((f"block_dk{dk}_g{gate}.o", os.path.join(CSRC, "swila_block_inst.cu"),
+                          [f"-DSWILA_DK={dk}", f"-DSWILA_GATE={gate}"]))
+        for bf16 in ((0, 1) if dk != 16 else ()):
+            units.append((f"tile_dk{dk}_b{bf16}.o", os.path.join(CSRC, "swila_tile_inst.cu"),
+                          [f"-DSWILA_DK={dk}", f"-DSWILA_BF16={bf16}"]))
     for f in sorted(os.listdir(CSRC)):  # any further stand-alone translation units
-        if f.endswith(".cu") and f not in ("swila_api.cu", "swila_scan_inst.cu"):
+        if f.endswith(".cu") and f not in ("swila_api.cu", "swila_scan_inst.cu", "swila_block_inst.cu", "swila_tile_inst.cu"):
             units.append((f[:-3] + ".o", os.path.join(CSRC, f), []))
     return units
 

@@ -24,6 +24,8 @@ int chunk_dispatch(const LaunchArgs &a);
 int chunk_gated_dispatch(LaunchArgs &a);
 int chunk_error_fetch(int *flag);
 int chunk_gated_error_fetch(int *flag);
+int block_dispatch_any(const LaunchArgs &a);
+int block_error_fetch(int *flag);
 
 static thread_local char g_cuda_err[256] = "";
 
@@ -188,6 +190,13 @@ static int run(const swila_shape_t *s, int T, const void *q, const void *k, cons
       a.algo = SWILA_ALGO_SCAN;
     }
   }
+  // What the chunked kernel does not cover, at the same length: the blocked scan (it and the sequential scan differ by
+  // rounding, so short prefills, which are continued by decode steps bit for bit, stay with the latter).
+  if (rc == -1000 && s->algo == SWILA_ALGO_AUTO && T >= 64) {
+    rc = block_dispatch_any(a);
+    if (rc == 0) return SWILA_OK;
+    if (rc != -1000) return cuda_fail((cudaError_t)rc);
+  }
 #define SWILA_CASE(DK)                                                                          \
   case DK:                                                                                      \
     if (a.gate_mode == 0) rc = scan_dispatch<DK, 0, false>(a);                                  \
@@ -249,6 +258,10 @@ int swila_device_status(void) {
   if (e != cudaSuccess) return cuda_fail(e);
   if (!flag) {
     e = (cudaError_t)chunk_gated_error_fetch(&flag);
+    if (e != cudaSuccess) return cuda_fail(e);
+  }
+  if (!flag) {
+    e = (cudaError_t)block_error_fetch(&flag);
     if (e != cudaSuccess) return cuda_fail(e);
   }
   if (flag) {  // (warp + 1) << 16 | low half of the barrier's shared-memory address; 1 if only a hand-over flag gave up

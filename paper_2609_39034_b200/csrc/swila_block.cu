@@ -1,0 +1,63 @@
+// Dispatch of the two kernels that evaluate several tokens at a time in FP32-grade arithmetic -- the register-tile kernel
+// (no decays, Dk = 64 and 128) and the blocked scan (the rest) -- and their error word.
+#include "swila_common.cuh"
+
+namespace swila {
+
+static __device__ int g_block_error = 0;
+
+#define SWILA_DECL(DK) \
+  template <> int block_dispatch<DK, 1>(const LaunchArgs &, int *, int); \
+  template <> int block_dispatch<DK, 2>(const LaunchArgs &, int *, int);
+SWILA_DECL(16)
+SWILA_DECL(64)
+SWILA_DECL(128)
+#undef SWILA_DECL
+template <> int block_dispatch<16, 0>(const LaunchArgs &, int *, int);
+template <> int tile_dispatch<64, false>(const LaunchArgs &, int *, int);
+template <> int tile_dispatch<64, true>(const LaunchArgs &, int *, int);
+template <> int tile_dispatch<128, false>(const LaunchArgs &, int *, int);
+template <> int tile_dispatch<128, true>(const LaunchArgs &, int *, int);
+
+// Returns a cudaError_t value (>= 0), or -1000 when the combination is not compiled (one decay per state element, or too
+// many components for the shared memory of the decayed operands).
+int block_dispatch_any(const LaunchArgs &a) {
+  static std::atomic<int *> err_of[kMaxDevices];
+  const int dev = current_device(), sms = sm_count();
+  int *err = dev >= 0 ? err_of[dev].load(std::memory_order_relaxed) : nullptr;
+  if (!err) {
+    const cudaError_t e = cudaGetSymbolAddress((void **)&err, g_block_error);
+    if (e != cudaSuccess) return (int)e;
+    if (dev >= 0) err_of[dev].store(err, std::memory_order_relaxed);
+  }
+  if (a.gate_mode == 0) {
+    // No decays: all components share their operands, and the products with the state go to the tensor pipe (measured at every
+    // shape tried, 1.05 to 2.3 times the blocked scan's pace).  At Dk = 16 there is nothing to contract: the serial part is all.
+    const bool bf16 = a.io_dtype == SWILA_IO_BF16;
+    if (a.Dk == 64) return bf16 ? tile_dispatch<64, true>(a, err, sms) : tile_dispatch<64, false>(a, err, sms);
+    if (a.Dk == 128) return bf16 ? tile_dispatch<128, true>(a, err, sms) : tile_dispatch<128, false>(a, err, sms);
+    return block_dispatch<16, 0>(a, err, sms);
+  }
+#define SWILA_CASE(DK)                                                     \
+  case DK:                                                                 \
+    if (a.gate_mode == 1) return block_dispatch<DK, 1>(a, err, sms);       \
+    if (a.gate_mode == 2) return block_dispatch<DK, 2>(a, err, sms);       \
+    return -1000;
+  switch (a.Dk) {
+    SWILA_CASE(16)
+    SWILA_CASE(64)
+    SWILA_CASE(128)
+    default: return -1000;
+  }
+#undef SWILA_CASE
+}
+
+// Reads (and clears) the error word of the current device; synchronises.
+int block_error_fetch(int *flag) {
+  int zero = 0;
+  cudaError_t e = cudaMemcpyFromSymbol(flag, g_block_error, sizeof(int));
+  if (e == cudaSuccess && *flag) e = cudaMemcpyToSymbol(g_block_error, &zero, sizeof(int));
+  return (int)e;
+}
+
+}  // namespace swila

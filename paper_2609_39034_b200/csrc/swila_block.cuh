@@ -1,0 +1,941 @@
+// Blocked scan of the SwiLA recurrence (Sec. 3.2, Eqs. 3.3-3.5) for sm_100a: full FP32 arithmetic, several tokens at a time.
+//
+// The sequential scan spends a token on two passes over the state with a reduction and the E-step between them, so a
+// warp mostly waits.  Here C tokens are taken together, exactly as the chunked tensor-core kernel does it:
+//
+//   p_t = W0.k_t, r_t = W0.q_t for the C tokens of a block             (dense, state in registers)
+//   token by token: delta = v - p_t, E-step, c_t; then p_t' += c_t k_t.k_t', r_t' += c_t k_t.q_t'   (scalars)
+//   W += sum_t c_t k_t                                                  (dense)
+//
+// -- the same recurrence, only the order of the additions differs.  All of it runs on the FP32 ALUs with FP32 operands, so
+// it serves what the kernels on the tensor pipe do not: decays per key dimension (every component has operands of its
+// own), decays per row outside the chunked kernel's coverage, and Dk = 16.
+//
+// A lane holds NC output columns of ONE component and L = DK / G of its key dimensions in registers (L * NC <= 128):
+// lane = (column group, component j, key slice g).  Then
+//  - a 16-byte operand load serves NC columns (16 packed FMAs at NC = 8): the loads of shared memory, of which each costs
+//    four cycles of the SM's load path, stay under half of the FMA time;
+//  - the reduction over the key slices is a butterfly that halves the columns each round and leaves NC / G columns per
+//    lane (12 shuffles for 16 values at G = 4).  A lane keeps its columns in the order i ^ mask(g), so that what it keeps
+//    and what it sends are fixed registers and no selection is needed;
+//  - the E-step is then evaluated once per row, not once per lane of a row.
+// Decays per key dimension make the operands of a component: prefix products times k and q for the predictions, suffix
+// products times k for the update, and Gram matrices per component.  Decays per row act on p, r and c as scalars.
+// Nothing is divided by a decay except in the per-component Gram matrices, which fall back to products when a block's
+// decays are so small that the quotients could overflow.
+//
+// Per block of tokens all threads convert the next but one block's k and q and form the next block's Gram matrices;
+// one thread issues the tensor copies (TMA) of what is to come.  One barrier per block (two with decays per key).
+#pragma once
+
+#include "swila_common.cuh"
+#include "swila_tma_maps.h"
+#include "swila_umma.cuh"
+
+namespace swila {
+
+template <typename IO_, int J_, int DK_, int NC_, int C_, int GATE_, bool EXT_>
+struct BlockCfg {
+  using IO = IO_;
+  static constexpr int J = J_, DK = DK_, NC = NC_, C = C_, GATE = GATE_;
+  static constexpr bool EXT = EXT_;  // the instantiation with the Temporal priors, r_debug and the statistics
+  static constexpr int ES = (int)sizeof(IO);
+  static constexpr int G = DK == 16 ? 1 : (DK == 64 ? (J <= 8 ? 4 : 2) : (J <= 4 ? 8 : (J == 8 ? 4 : 2)));
+  static constexpr int L = DK / G;
+  static constexpr int CG = 32 / (G * J);     // column groups per warp
+  static constexpr int CPW = CG * NC;         // columns per warp
+  static constexpr int OC = NC / G;           // columns per lane after the reduction
+  static constexpr int GJ = GATE == 1 ? J : 1;  // operand sets: one per component with decays per key dimension
+  static_assert(G * J * CG == 32 && L % 4 == 0 && (OC == 1 || OC == 2) && OC * G == NC && L * NC <= 128, "lane split");
+  static constexpr int PAD = 16 / ES;         // gate rows are fetched this much wider: rows of components skewed by a bank group
+  // floats; the skew of 16 between components keeps the two that share a quarter warp apart (G = 4)
+  static constexpr int KQ = 2 * C * DK;                                        // converted k and q of a block: k_t, q_t alternating
+  static constexpr int KT = GATE == 1 ? 2 * C * DK + 16 : 0, KB = GATE == 1 ? C * DK + 16 : 0, AC = GATE == 1 ? DK + 16 : 0;
+  static constexpr int GR = C * 2 * C + 4;                                      // Gram rows [s][k.k_t | k.q_t] of one operand set
+  static constexpr int NKQ = GATE == 1 ? 2 : 3;                                 // ring of converted blocks
+  static constexpr int RW = CG * J * NC;                                        // rows per warp
+  static constexpr int NCOPY = OC == 1 ? 2 : 1;                                 // orders the coefficients are stored in
+  // a warp's exchange buffer, floats: first every lane's p_t, r_t, then the update coefficients of the warp's rows
+  static constexpr int CB1 = (C + (GATE == 2 ? 1 : 0)) * NCOPY * RW * 2, CB2 = C * 2 * OC * 32;
+  static constexpr int CB = CB1 > CB2 ? CB1 : CB2;
+};
+
+__host__ __device__ constexpr int block_up128(int n) { return (n + 127) & ~127; }
+
+// Shared-memory map of a launch (bytes); the number of columns per thread block is a launch parameter.
+struct BlockSmem {
+  int rawkq, rawkq_stage, alpha, alpha_stage, gates, gates_stage, g_be, g_pk, g_pq, g_gk, g_gq, g_ar, kq, kt, kb, kh, ac, gram, cbuf, ost, bars, total;
+};
+template <class Cf>
+__host__ __device__ inline BlockSmem block_smem(int nwarps, bool temporal, bool row_alpha) {
+  BlockSmem m;
+  const int cols = nwarps * Cf::CPW, grow = cols + Cf::PAD;
+  const int gate = block_up128(Cf::C * Cf::J * grow * Cf::ES), vec = block_up128(Cf::C * cols * Cf::ES);
+  int off = 0;
+  m.rawkq = off; m.rawkq_stage = 2 * block_up128(Cf::C * Cf::DK * Cf::ES); off += 2 * m.rawkq_stage;
+  m.alpha = off; m.alpha_stage = Cf::GATE == 1 ? Cf::C * Cf::J * Cf::DK * 4 : 0; off += 2 * m.alpha_stage;
+  m.gates = off;
+  m.g_be = vec; m.g_pk = m.g_be + gate; m.g_pq = m.g_pk + gate; m.g_gk = m.g_pq + gate;
+  m.g_gq = m.g_gk + (temporal ? vec : 0); m.g_ar = m.g_gq + (temporal ? vec : 0);
+  m.gates_stage = m.g_ar + (row_alpha ? block_up128(Cf::C * Cf::J * (cols + 4) * 4) : 0);
+  off += 2 * m.gates_stage;
+  m.kq = off; off += Cf::NKQ * Cf::KQ * 4;
+  m.kt = off; off += 2 * Cf::J * Cf::KT * 4;
+  m.kb = off; off += 2 * Cf::J * Cf::KB * 4;
+  m.kh = off; off += Cf::J * Cf::KB * 4;
+  m.ac = off; off += 2 * Cf::J * Cf::AC * 4;
+  m.gram = off; off += 2 * Cf::GJ * Cf::GR * 4;
+  m.cbuf = off; off += nwarps * Cf::CB * 4;
+  m.ost = off; off += block_up128(nwarps * Cf::C * Cf::CPW * Cf::ES);
+  m.bars = off; off += 64;
+  m.total = off + 128;  // the kernel aligns its window to 128 bytes
+  return m;
+}
+
+// Tensor maps of a launch: boxes of C tokens.
+struct BlockMaps {
+  CUtensorMap k, q, v, be, pk, pq, gk, gq, al;
+};
+
+// Bounded wait (two seconds of wall time); on expiry the error word is set and every later wait of the thread is skipped.
+static __device__ __noinline__ bool block_wait_poll(uint64_t *bar, uint32_t parity, int *err) {
+  const unsigned long long t0 = umma::global_timer_ns();
+#pragma unroll 1
+  for (uint32_t i = 1;; ++i) {
+    if (umma::mbar_try_wait(bar, parity)) return true;
+    if ((i & 255u) == 0 && umma::global_timer_ns() - t0 > 2000000000ull) {
+      atomicCAS(err, 0, (int)(((threadIdx.x >> 5) + 1) * 65536 + (umma::smem_u32(bar) & 0xffffu)));
+      return false;
+    }
+  }
+}
+
+// Barrier and OR over the `n` preparing threads.
+__device__ __forceinline__ int named_bar_or(int n, bool x) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %2, 0;\n\tbarrier.cta.red.or.pred q, 1, %1, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+      : "=r"(r) : "r"(n), "r"((unsigned)x) : "memory");
+  return r;
+}
+
+// OC consecutive values of the io dtype
+template <typename IO, int OC>
+__device__ __forceinline__ void block_ld(const IO *p, float (&x)[OC]) {
+  if constexpr (OC % 2 == 0 && sizeof(IO) == 2) {
+#pragma unroll
+    for (int o = 0; o < OC; o += 2) {
+      const uint32_t u = *reinterpret_cast<const uint32_t *>(p + o);
+      x[o] = __uint_as_float(u << 16);
+      x[o + 1] = __uint_as_float(u & 0xffff0000u);
+    }
+  } else if constexpr (OC % 2 == 0) {
+#pragma unroll
+    for (int o = 0; o < OC; o += 2) {
+      const float2 u = *reinterpret_cast<const float2 *>(p + o);
+      x[o] = u.x; x[o + 1] = u.y;
+    }
+  } else {
+#pragma unroll
+    for (int o = 0; o < OC; ++o) x[o] = to_f32(p[o]);
+  }
+}
+
+// ---- preparation phases, all threads of the block ------------------------------------------
+// k and q of one block as FP32 vectors, k_t and q_t alternating; with qkv_act after SiLU and the L2 norm over the key
+// dimension (App. B.2, App. D.1): the DK / 4 work items of a vector are adjacent lanes of one warp.
+template <class Cf>
+__device__ __forceinline__ void block_convert(const unsigned char *raw, int half, float *kq, bool act, int tid, int nt) {
+  using IO = typename Cf::IO;
+  constexpr int DK = Cf::DK, C = Cf::C, LPT = DK / 4;
+  for (int i = tid; i < 2 * C * LPT; i += nt) {  // whole warps run a trip or none: the item count is a multiple of 32
+    const int isq = i >= C * LPT, e = i - isq * C * LPT, t = e / LPT, d = (e - t * LPT) * 4;
+    const IO *src = reinterpret_cast<const IO *>(raw + isq * half) + t * DK + d;
+    float x[4];
+    if constexpr (sizeof(IO) == 2) {
+      const uint2 u = *reinterpret_cast<const uint2 *>(src);
+      x[0] = __uint_as_float(u.x << 16); x[1] = __uint_as_float(u.x & 0xffff0000u);
+      x[2] = __uint_as_float(u.y << 16); x[3] = __uint_as_float(u.y & 0xffff0000u);
+    } else {
+      const float4 u = *reinterpret_cast<const float4 *>(src);
+      x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
+    }
+    if (act) {
+#pragma unroll
+      for (int n = 0; n < 4; ++n) x[n] = silu_approx(x[n]);
+      float ss = x[0] * x[0] + x[1] * x[1] + x[2] * x[2] + x[3] * x[3];
+#pragma unroll
+      for (int off = 1; off < LPT; off <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+      const float inv = rsqrtf(ss + kL2Eps);
+#pragma unroll
+      for (int n = 0; n < 4; ++n) x[n] *= inv;
+    }
+    *reinterpret_cast<float4 *>(kq + (2 * t + isq) * DK + d) = make_float4(x[0], x[1], x[2], x[3]);
+  }
+}
+
+// Decays per key dimension, one block: per component the prediction and readout operands A_t k_t, A_t q_t (A_t = product of
+// the decays up to token t; the post-decay form of Eq. 3.7 predicts with A_{t-1}), the update operands
+// (product of the later decays) k_t, the whole product, and k_t / A_t for the Gram matrices.  Returns whether some product is
+// too small for that quotient.  A thread takes one component and two key dimensions.
+template <class Cf>
+__device__ __forceinline__ bool block_decay(const float *kq, const float *alpha, float *kt, float *kb, float *kh, float *ac, int nvalid,
+                                            bool post, int tid, int nt) {
+  constexpr int DK = Cf::DK, C = Cf::C, J = Cf::J;
+  bool tiny = false;
+  for (int i = tid; i < J * DK / 2; i += nt) {
+    const int j = i / (DK / 2), d = (i - j * (DK / 2)) * 2;
+    float2 a[C], k[C];
+#pragma unroll
+    for (int t = 0; t < C; ++t) {
+      a[t] = *reinterpret_cast<const float2 *>(alpha + (t * J + j) * DK + d);
+      if (t >= nvalid) a[t] = make_float2(1.f, 1.f);  // past the end of the sequence
+      k[t] = *reinterpret_cast<const float2 *>(kq + 2 * t * DK + d);
+    }
+    float2 A = make_float2(1.f, 1.f), S = A;
+    float *kto = kt + j * Cf::KT + d, *kho = kh + j * Cf::KB + d, *kbo = kb + j * Cf::KB + d;
+#pragma unroll
+    for (int t = 0; t < C; ++t) {
+      const float2 q = *reinterpret_cast<const float2 *>(kq + (2 * t + 1) * DK + d);
+      const float2 before = A;
+      A = mul2(A, a[t]);
+      *reinterpret_cast<float2 *>(kto + 2 * t * DK) = mul2(post ? before : A, k[t]);
+      *reinterpret_cast<float2 *>(kto + (2 * t + 1) * DK) = mul2(A, q);
+      *reinterpret_cast<float2 *>(kho + t * DK) = make_float2(k[t].x * rcp_approx(A.x), k[t].y * rcp_approx(A.y));
+    }
+    tiny = tiny || !(fminf(A.x, A.y) > 1e-18f);
+#pragma unroll
+    for (int t = C - 1; t >= 0; --t) {
+      *reinterpret_cast<float2 *>(kbo + t * DK) = mul2(S, k[t]);
+      S = mul2(S, a[t]);
+    }
+    *reinterpret_cast<float2 *>(ac + j * Cf::AC + d) = S;
+  }
+  return tiny;
+}
+
+// Gram rows of one block: gram[s][t] = u_s.kv_t for t > s and gram[s][C + t] = u_s.qv_t for t >= s, the vectors kv_t, qv_t
+// alternating in `vec`, u_s at stride us.  Four lanes share the key dimensions of a 2 x 2 tile (two s, the k and q of one t).
+template <class Cf>
+__device__ __forceinline__ void block_gram(const float *u, int us, int ucomp, const float *vec, int vcomp, float *gram, int tid, int nt) {
+  constexpr int DK = Cf::DK, C = Cf::C;
+  constexpr int NI = C == 8 ? 20 : 6;  // tiles (pair of s, t) with t >= the first s of the pair
+  constexpr int TOTAL = NI * 4 * Cf::GJ;
+  static_assert(C == 8 || C == 4, "tile table");
+  for (int i0 = 0; i0 < TOTAL; i0 += nt) {
+    const int it = min(i0 + (tid & ~3), TOTAL - 4) + (tid & 3);  // every lane takes part in the shuffles (the last tile may be formed twice)
+    const int kd = it & 3, rest = it >> 2, jj = rest / NI, n = rest - jj * NI;
+    int sp, t;
+    if constexpr (C == 8) {
+      sp = n < 8 ? 0 : (n < 14 ? 1 : (n < 18 ? 2 : 3));
+      t = n < 8 ? n : (n < 14 ? n - 6 : (n < 18 ? n - 10 : n - 12));
+    } else {
+      sp = n < 4 ? 0 : 1;
+      t = n < 4 ? n : n - 2;
+    }
+    const float *s0 = u + jj * ucomp + 2 * sp * us + kd * 4, *s1 = s0 + us;
+    const float *kv = vec + jj * vcomp + 2 * t * DK + kd * 4, *qv = kv + DK;
+    float2 d[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) d[x] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < DK / 16; ++i) {
+      const float4 a = *reinterpret_cast<const float4 *>(s0 + i * 16), b = *reinterpret_cast<const float4 *>(s1 + i * 16);
+      const float4 k4 = *reinterpret_cast<const float4 *>(kv + i * 16), q4 = *reinterpret_cast<const float4 *>(qv + i * 16);
+      d[0] = fma2(make_float2(a.x, a.y), make_float2(k4.x, k4.y), d[0]); d[0] = fma2(make_float2(a.z, a.w), make_float2(k4.z, k4.w), d[0]);
+      d[1] = fma2(make_float2(a.x, a.y), make_float2(q4.x, q4.y), d[1]); d[1] = fma2(make_float2(a.z, a.w), make_float2(q4.z, q4.w), d[1]);
+      d[2] = fma2(make_float2(b.x, b.y), make_float2(k4.x, k4.y), d[2]); d[2] = fma2(make_float2(b.z, b.w), make_float2(k4.z, k4.w), d[2]);
+      d[3] = fma2(make_float2(b.x, b.y), make_float2(q4.x, q4.y), d[3]); d[3] = fma2(make_float2(b.z, b.w), make_float2(q4.z, q4.w), d[3]);
+    }
+    float g[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      g[x] = d[x].x + d[x].y;
+      g[x] += __shfl_xor_sync(0xffffffffu, g[x], 1);
+      g[x] += __shfl_xor_sync(0xffffffffu, g[x], 2);
+    }
+    const float mine = kd == 0 ? g[0] : (kd == 1 ? g[1] : (kd == 2 ? g[2] : g[3]));
+    gram[jj * Cf::GR + (2 * sp + (kd >> 1)) * 2 * C + (kd & 1) * C + t] = mine;
+  }
+}
+
+// The same with the decays multiplied out between s and t: exact for any decay, zero included.  Rare, so not optimised.
+template <class Cf>
+__device__ __noinline__ void block_gram_products(const float *kq, const float *alpha, float *gram, int nvalid, bool post, int tid, int nt) {
+  constexpr int DK = Cf::DK, C = Cf::C, J = Cf::J;
+  for (int it = tid; it < J * C * C; it += nt) {
+    const int j = it / (C * C), s = (it / C) % C, t = it % C;
+    if (t < s) continue;
+    float gk = 0.f, gq = 0.f;
+    for (int d = 0; d < DK; ++d) {
+      float x = kq[2 * s * DK + d], xk = x;
+      for (int m = s + 1; m <= t; ++m) {
+        xk = x;
+        if (m < nvalid) x *= alpha[(m * J + j) * DK + d];
+      }
+      gk = fmaf(post ? xk : x, kq[2 * t * DK + d], gk);
+      gq = fmaf(x, kq[(2 * t + 1) * DK + d], gq);
+    }
+    gram[j * Cf::GR + s * 2 * C + t] = gk;
+    gram[j * Cf::GR + s * 2 * C + C + t] = gq;
+  }
+}
+
+// ---- the scalar part of a block: one lane, OC columns of one component -----------------------
+template <class Cf>
+struct BlockLane {
+  int j, g, cg, mask;  // component, key slice, column group, column order of the registers
+  int lc;              // first owned column inside the thread block's slice
+  float rp[Cf::OC], rho[Cf::OC];                       // Temporal: carried distributions
+  float s_r[Cf::OC], s_rh[Cf::OC], s_q[Cf::OC], s_qh[Cf::OC];  // statistics (entropies in bits)
+};
+
+// Sum over the J lanes of a column (distance G).
+template <class Cf>
+__device__ __forceinline__ float block_sum_j(float x) {
+  if constexpr (Cf::J == 4) {  // three independent shuffles: shorter than two dependent rounds
+    const float a = __shfl_xor_sync(0xffffffffu, x, Cf::G), b = __shfl_xor_sync(0xffffffffu, x, 2 * Cf::G);
+    const float c = __shfl_xor_sync(0xffffffffu, x, 3 * Cf::G);
+    return (x + a) + (b + c);
+  } else {
+#pragma unroll
+    for (int off = 1; off < Cf::J; off <<= 1) x += __shfl_xor_sync(0xffffffffu, x, off * Cf::G);
+    return x;
+  }
+}
+template <class Cf>
+__device__ __forceinline__ float block_max_j(float x) {
+#pragma unroll
+  for (int off = 1; off < Cf::J; off <<= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, off * Cf::G));
+  return x;
+}
+
+// Entered with the lane's p_t and r_t of the block in `xch` ([t][lane][p of OC columns, r of OC columns]); hands every update
+// coefficient to put(t, o, c) and writes the outputs to `ost` ([C][CPW], io dtype).  EXACT subtracts the maximum before every exponential; without it the pass
+// returns true when a normaliser left the safe range, and the caller runs the block again.
+template <class Cf, bool EXACT, class Put>
+__device__ __forceinline__ bool block_tokens(const ScanParams &p, const BlockSmem &m, BlockLane<Cf> &ln, const float *xch, Put put,
+                                             const unsigned char *gates, const float *gram, typename Cf::IO *ost, int cols, int nvalid, int col,
+                                             size_t tok) {
+  using IO = typename Cf::IO;
+  constexpr int J = Cf::J, C = Cf::C, OC = Cf::OC, G = Cf::G;
+  const int grow = cols + Cf::PAD;
+  const bool temporal = Cf::EXT && p.temporal != 0;
+  const IO *gv = reinterpret_cast<const IO *>(gates) + ln.lc;
+  const IO *gbe = reinterpret_cast<const IO *>(gates + m.g_be) + ln.j * grow + ln.lc;
+  const IO *gpk = reinterpret_cast<const IO *>(gates + m.g_pk) + ln.j * grow + ln.lc;
+  const IO *gpq = reinterpret_cast<const IO *>(gates + m.g_pq) + ln.j * grow + ln.lc;
+  [[maybe_unused]] const IO *ggk = reinterpret_cast<const IO *>(gates + m.g_gk) + ln.lc;
+  [[maybe_unused]] const IO *ggq = reinterpret_cast<const IO *>(gates + m.g_gq) + ln.lc;
+  [[maybe_unused]] const float *gar = reinterpret_cast<const float *>(gates + m.g_ar) + ln.j * (cols + 4) + ln.lc;
+  auto P = [&](float2(&x)[OC][C / 2], int o, int t) -> float & { return (t & 1) ? x[o][t >> 1].y : x[o][t >> 1].x; };
+  float2 P2[OC][C / 2], R2[OC][C / 2];
+#pragma unroll
+  for (int t = 0; t < C; ++t) {
+    float x[2 * OC];
+    if constexpr (OC == 1) {
+      const float2 y = *reinterpret_cast<const float2 *>(xch + t * 64);
+      x[0] = y.x; x[1] = y.y;
+    } else {
+#pragma unroll
+      for (int i = 0; i < OC / 2; ++i) {
+        const float4 y = *reinterpret_cast<const float4 *>(xch + t * 64 * OC + 4 * i);
+        x[4 * i] = y.x; x[4 * i + 1] = y.y; x[4 * i + 2] = y.z; x[4 * i + 3] = y.w;
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < OC; ++o) { P(P2, o, t) = x[o]; P(R2, o, t) = x[OC + o]; }
+  }
+  __syncwarp();  // the buffer is about to take the coefficients
+  bool bad = false;
+  float rp[OC], s_r[OC], s_rh[OC];
+#pragma unroll
+  for (int o = 0; o < OC; ++o) { rp[o] = ln.rp[o]; s_r[o] = s_rh[o] = 0.f; }
+
+  float v[C][OC];
+#pragma unroll
+  for (int t = 0; t < C; ++t) block_ld<IO, OC>(gv + t * cols, v[t]);
+  if (p.qkv_act) {
+#pragma unroll
+    for (int t = 0; t < C; ++t)
+#pragma unroll
+      for (int o = 0; o < OC; ++o) v[t][o] = silu_approx(v[t][o]);
+  }
+
+#pragma unroll
+  for (int t = 0; t < C; ++t) {
+    float be[OC], lk[OC];
+    block_ld<IO, OC>(gbe + t * J * grow, be);
+    block_ld<IO, OC>(gpk + t * J * grow, lk);
+    [[maybe_unused]] float ar[OC];
+    if constexpr (Cf::GATE == 2) {
+      // one decay per row: everything that is still to be used is decayed as the state would be
+      if (p.gran == SWILA_GATE_PER_OUT) {
+        block_ld<float, OC>(gar + t * J * (cols + 4), ar);
+      } else {
+        const float a = t < nvalid ? __ldg(p.alpha + (tok + t) * J + ln.j) : 1.f;
+#pragma unroll
+        for (int o = 0; o < OC; ++o) ar[o] = a;
+      }
+#pragma unroll
+      for (int o = 0; o < OC; ++o) {
+        if (t >= nvalid) ar[o] = 1.f;
+        if (!p.post) P(P2, o, t) *= ar[o];
+      }
+    }
+    float e[OC], c[OC];
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      be[o] = sigmoid_approx(be[o]);
+      if (t >= nvalid) be[o] = 0.f;  // past the end of the sequence: no update
+      const float delta = v[t][o] - P(P2, o, t);
+      float a;
+      if (temporal) {
+        // prior (1 - g) r_{t-1} + g pi^k, pi^k normalised (App. B.3)
+        const float x = lk[o] * kLog2e, ex = ex2_approx(x - block_max_j<Cf>(x));
+        const float pk = ex * rcp_approx(block_sum_j<Cf>(ex));
+        float gk[OC];
+        block_ld<IO, OC>(ggk + t * cols, gk);
+        const float prior = fmaf(sigmoid_approx(gk[o]), pk - rp[o], rp[o]);
+        a = fmaf(-kHalfLog2e * delta, delta, lg2_approx(prior));
+      } else {
+        a = fmaf(-kHalfLog2e * delta, delta, lk[o] * kLog2e);
+      }
+      if constexpr (EXACT) a -= block_max_j<Cf>(a);
+      e[o] = ex2_approx(a);
+      const float sum = block_sum_j<Cf>(e[o]);
+      if constexpr (!EXACT) bad = bad || !(sum > 1e-30f && sum < 1e30f);
+      const float rs = rcp_approx(sum);
+      c[o] = ((be[o] * delta) * e[o]) * rs;
+      if constexpr (Cf::EXT) {
+        const float r = e[o] * rs;
+        if (t < nvalid) {
+          rp[o] = r;
+          s_r[o] += r;
+          if (r > 0.f) s_rh[o] = fmaf(r, lg2_approx(e[o]) - lg2_approx(sum), s_rh[o]);
+          if (p.r_debug && col + o < p.Dv) p.r_debug[((tok + t) * J + ln.j) * p.Dv + col + o] = r;
+        }
+      }
+    }
+    if constexpr (Cf::GATE == 2) {
+#pragma unroll
+      for (int o = 0; o < OC; ++o) {
+#pragma unroll
+        for (int u = t + 1; u < C; ++u) P(P2, o, u) *= ar[o];
+#pragma unroll
+        for (int u = t; u < C; ++u) P(R2, o, u) *= ar[o];
+      }
+    }
+    // pushes into the later predictions and into the readouts from this token on
+    const float4 *gr = reinterpret_cast<const float4 *>(gram + t * 2 * C);
+    float gk[C], gq[C];
+#pragma unroll
+    for (int i = 0; i < C / 4; ++i) {
+      if (4 * i + 3 > t) {
+        const float4 x = gr[i];
+        gk[4 * i] = x.x; gk[4 * i + 1] = x.y; gk[4 * i + 2] = x.z; gk[4 * i + 3] = x.w;
+      }
+      if (4 * i + 3 >= t) {
+        const float4 x = gr[C / 4 + i];
+        gq[4 * i] = x.x; gq[4 * i + 1] = x.y; gq[4 * i + 2] = x.z; gq[4 * i + 3] = x.w;
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      put(t, o, c[o]);
+      const float2 c2 = make_float2(c[o], c[o]);
+      if ((t & 1) == 0) P(P2, o, t + 1) = fmaf(c[o], gk[t + 1], P(P2, o, t + 1));
+#pragma unroll
+      for (int u = t / 2 + 1; u < C / 2; ++u) P2[o][u] = fma2(c2, make_float2(gk[2 * u], gk[2 * u + 1]), P2[o][u]);
+      if (t & 1) P(R2, o, t) = fmaf(c[o], gq[t], P(R2, o, t));
+#pragma unroll
+      for (int u = (t + 1) / 2; u < C / 2; ++u) R2[o][u] = fma2(c2, make_float2(gq[2 * u], gq[2 * u + 1]), R2[o][u]);
+    }
+  }
+
+  // ---- readouts: o_t = sum_j pi^q_j (w_t.q_t)_j ----
+  constexpr int N = C * OC;
+  float num[N], den[N];
+  [[maybe_unused]] float rho[OC], s_q[OC], s_qh[OC];
+#pragma unroll
+  for (int o = 0; o < OC; ++o) { rho[o] = ln.rho[o]; s_q[o] = s_qh[o] = 0.f; }
+#pragma unroll
+  for (int t = 0; t < C; ++t) {
+    float x[OC];
+    block_ld<IO, OC>(gpq + t * J * grow, x);
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      x[o] *= kLog2e;
+      if (EXACT || temporal) x[o] -= block_max_j<Cf>(x[o]);
+      const float e = J == 1 ? 1.f : ex2_approx(x[o]);
+      num[t * OC + o] = e * P(R2, o, t);
+      den[t * OC + o] = e;
+      if constexpr (Cf::EXT) {
+        float w = 0.f;
+        if (temporal) {
+          w = e * rcp_approx(block_sum_j<Cf>(e));
+          float gq[OC];
+          block_ld<IO, OC>(ggq + t * cols, gq);
+          if (t < nvalid) rho[o] = fmaf(sigmoid_approx(gq[o]), w - rho[o], rho[o]);
+          w = rho[o];
+          num[t * OC + o] = w * P(R2, o, t);
+        } else if (p.rho_sum || p.rho_ent) {
+          w = e * rcp_approx(block_sum_j<Cf>(e));
+        }
+        if ((p.rho_sum || p.rho_ent) && t < nvalid) {
+          s_q[o] += w;
+          if (w > 0.f) s_qh[o] = fmaf(w, lg2_approx(w), s_qh[o]);
+        }
+      }
+    }
+  }
+  // sums over the J lanes of a column.  With at least J values per lane each lane ends up with N / J of the sums: half of
+  // the values change lanes each round.
+  constexpr bool SCATTER = N >= J;
+  if constexpr (SCATTER) {
+#pragma unroll
+    for (int h = N / 2, d = J / 2; d >= 1; h /= 2, d /= 2) {
+      const bool up = (ln.j & d) != 0;
+#pragma unroll
+      for (int n = 0; n < N / 2; ++n) {
+        if (n < h) {
+          const float kn = up ? num[n + h] : num[n], sn = up ? num[n] : num[n + h];
+          num[n] = kn + __shfl_xor_sync(0xffffffffu, sn, d * G);
+          if (!temporal) {
+            const float kd = up ? den[n + h] : den[n], sd = up ? den[n] : den[n + h];
+            den[n] = kd + __shfl_xor_sync(0xffffffffu, sd, d * G);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int n = 0; n < N / J; ++n) {
+      const int idx = ln.j * (N / J) + n, t = idx / OC, o = idx - t * OC;
+      const float out = temporal ? num[n] : (J == 1 ? num[n] : num[n] * rcp_approx(den[n]));
+      if constexpr (!EXACT) bad = bad || (!temporal && !(den[n] > 1e-30f && den[n] < 1e30f));
+      from_f32(ost[t * Cf::CPW + ln.cg * Cf::NC + ln.mask + o], out);
+    }
+  } else {
+#pragma unroll
+    for (int n = 0; n < N; ++n) {
+      num[n] = block_sum_j<Cf>(num[n]);
+      if (!temporal) den[n] = block_sum_j<Cf>(den[n]);
+      if constexpr (!EXACT) bad = bad || (!temporal && !(den[n] > 1e-30f && den[n] < 1e30f));
+      if (ln.j == n) from_f32(ost[(n / OC) * Cf::CPW + ln.cg * Cf::NC + ln.mask + n % OC], temporal ? num[n] : num[n] * rcp_approx(den[n]));
+    }
+  }
+  if constexpr (!EXACT) {
+    if (__any_sync(0xffffffffu, bad)) return true;
+  }
+  if constexpr (Cf::EXT) {  // this pass stands
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      ln.rp[o] = rp[o]; ln.rho[o] = rho[o];
+      ln.s_r[o] += s_r[o]; ln.s_rh[o] += s_rh[o]; ln.s_q[o] += s_q[o]; ln.s_qh[o] += s_qh[o];
+    }
+  }
+  return false;
+}
+
+// ---- the kernel ---------------------------------------------------------------------------
+template <class Cf>
+__global__ void __launch_bounds__(256, Cf::L *Cf::NC <= 64 ? 2 : 1)
+    swila_block_kernel(const __grid_constant__ ScanParams p, const __grid_constant__ BlockMaps maps, const int nwarps, int *err) {
+  using IO = typename Cf::IO;
+  using namespace umma;
+  constexpr int J = Cf::J, DK = Cf::DK, C = Cf::C, G = Cf::G, L = Cf::L, NC = Cf::NC, OC = Cf::OC, CPW = Cf::CPW, GATE = Cf::GATE;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *smem = smem_raw + ((128u - (smem_u32(smem_raw) & 127u)) & 127u);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // `nwarps` warps hold the state; warps beyond them, if any, prepare the operands (else the state warps do)
+  const int pw0 = (int)(blockDim.x >> 5) > nwarps ? nwarps : 0;
+  const bool holds = warp < nwarps, prepares = warp >= pw0;
+  const int ptid = tid - pw0 * 32, nt = blockDim.x - pw0 * 32;
+  const int cols = nwarps * CPW;
+  const bool temporal = Cf::EXT && p.temporal != 0;
+  const bool row_alpha = GATE == 2 && p.gran == SWILA_GATE_PER_OUT;
+  const BlockSmem m = block_smem<Cf>(nwarps, temporal, row_alpha);
+  const int nslice = (p.Dv + cols - 1) / cols;
+  const int bh = blockIdx.x / nslice, col0 = (blockIdx.x - bh * nslice) * cols;
+  const size_t tok0 = (size_t)bh * p.T;
+  const int nb = (p.T + C - 1) / C;
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + m.bars);  // k, q [2]; gates [2]; decays [2]
+  float *kq_all = reinterpret_cast<float *>(smem + m.kq);
+  float *gram_all = reinterpret_cast<float *>(smem + m.gram);
+
+  BlockLane<Cf> ln;
+  ln.g = lane % G; ln.j = (lane / G) % J; ln.cg = lane / (G * J);
+  ln.mask = ln.g * OC;  // bit r of g (from the top) says which half of the columns the lane keeps in round r
+  ln.lc = warp * CPW + ln.cg * NC + ln.mask;
+  const int j = ln.j, g = ln.g, mask = ln.mask;
+  const int colw = col0 + warp * CPW + ln.cg * NC;  // first column of the lane's group
+#pragma unroll
+  for (int o = 0; o < OC; ++o) {
+    ln.rp[o] = ln.rho[o] = 1.0f / J;
+    ln.s_r[o] = ln.s_rh[o] = ln.s_q[o] = ln.s_qh[o] = 0.f;
+    if (temporal && holds && colw + mask + o < p.Dv) {
+      const size_t at = ((size_t)bh * J + j) * p.Dv + colw + mask + o;
+      if (p.r_in) ln.rp[o] = p.r_in[at];
+      if (p.rho_in) ln.rho[o] = p.rho_in[at];
+    }
+  }
+
+  if (tid == 0) {
+    for (int i = 0; i < 6; ++i) mbar_init(&bars[i], 1);
+    mbar_fence_init();
+  }
+  __syncthreads();
+  // tensor copies of block b; the buffers were last read through ordinary loads, hence the proxy fence
+  auto load_kq = [&](int b) {
+    unsigned char *dst = smem + m.rawkq + (b & 1) * m.rawkq_stage;
+    mbar_arrive_expect_tx(&bars[b & 1], 2 * C * DK * Cf::ES);
+    tma_load_3d(dst, &maps.k, 0, b * C, bh, &bars[b & 1]);
+    tma_load_3d(dst + m.rawkq_stage / 2, &maps.q, 0, b * C, bh, &bars[b & 1]);
+  };
+  auto load_gates = [&](int b) {
+    unsigned char *dst = smem + m.gates + (b & 1) * m.gates_stage;
+    uint64_t *bar = &bars[2 + (b & 1)];
+    const int vec = C * cols * Cf::ES, gate = C * J * (cols + Cf::PAD) * Cf::ES;
+    mbar_arrive_expect_tx(bar, vec * (temporal ? 3 : 1) + 3 * gate + (row_alpha ? C * J * (cols + 4) * 4 : 0));
+    tma_load_3d(dst, &maps.v, col0, b * C, bh, bar);
+    tma_load_4d(dst + m.g_be, &maps.be, col0, 0, b * C, bh, bar);
+    tma_load_4d(dst + m.g_pk, &maps.pk, col0, 0, b * C, bh, bar);
+    tma_load_4d(dst + m.g_pq, &maps.pq, col0, 0, b * C, bh, bar);
+    if (temporal) {
+      tma_load_3d(dst + m.g_gk, &maps.gk, col0, b * C, bh, bar);
+      tma_load_3d(dst + m.g_gq, &maps.gq, col0, b * C, bh, bar);
+    }
+    if (row_alpha) tma_load_4d(dst + m.g_ar, &maps.al, col0, 0, b * C, bh, bar);
+  };
+  auto load_alpha = [&](int b) {
+    mbar_arrive_expect_tx(&bars[4 + (b & 1)], m.alpha_stage);
+    tma_load_4d(smem + m.alpha + (b & 1) * m.alpha_stage, &maps.al, 0, 0, b * C, bh, &bars[4 + (b & 1)]);
+  };
+  bool failed = false;
+  auto wait = [&](int which, int b) {
+    uint64_t *bar = &bars[which + (b & 1)];
+    if (!failed && !mbar_try_wait(bar, (b >> 1) & 1) && !block_wait_poll(bar, (b >> 1) & 1, err)) failed = true;
+  };
+  if (ptid == 0) load_kq(0);
+
+  // ---- state -> registers: register i of a lane holds column i ^ mask of its group, key dims (n*G + g)*4 .. +3 ----
+  float2 w[NC][L / 2];
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    const int col = colw + (i ^ mask);
+    const float *src = (p.W_in && holds && col < p.Dv) ? p.W_in + (((size_t)bh * J + j) * p.Dv + col) * DK : nullptr;
+#pragma unroll
+    for (int n = 0; n < L / 4; ++n) {
+      float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (src) t = __ldcs(reinterpret_cast<const float4 *>(src + (n * G + g) * 4));
+      w[i][2 * n] = make_float2(t.x, t.y);
+      w[i][2 * n + 1] = make_float2(t.z, t.w);
+    }
+  }
+
+  // Iteration b: convert block b+2, Gram matrices of block b+1 (decayed operands before that, GATE 1), then block b itself.
+#pragma unroll 1
+  for (int b = -2; b < nb; ++b) {
+    if (ptid == 0) {
+      fence_async_smem();
+      if (b + 3 < nb) load_kq(b + 3);
+      if (b + 1 >= 0 && b + 1 < nb) load_gates(b + 1);
+      if constexpr (GATE == 1) {
+        if (b + 2 < nb) load_alpha(b + 2);
+      }
+    }
+    const int b1 = b + 1;
+    const bool prep = b1 >= 0 && b1 < nb;
+    const int nv1 = min(C, p.T - b1 * C);
+    float *kq1 = kq_all + (b1 % Cf::NKQ) * Cf::KQ;  // (not used for b1 < 0)
+    int slow = 0;
+    if constexpr (GATE == 1) {
+      bool tiny = false;
+      if (prep && prepares) {
+        wait(4, b1);
+        tiny = block_decay<Cf>(kq1, reinterpret_cast<const float *>(smem + m.alpha + (b1 & 1) * m.alpha_stage),
+                               reinterpret_cast<float *>(smem + m.kt) + (b1 & 1) * J * Cf::KT, reinterpret_cast<float *>(smem + m.kb) + (b1 & 1) * J * Cf::KB,
+                               reinterpret_cast<float *>(smem + m.kh), reinterpret_cast<float *>(smem + m.ac) + (b1 & 1) * J * Cf::AC, nv1, p.post, ptid, nt);
+      }
+      if (prepares) slow = pw0 ? named_bar_or(nt, tiny) : __syncthreads_or(tiny);
+    }
+    if (prepares && b + 2 < nb) {
+      wait(0, b + 2);
+      block_convert<Cf>(smem + m.rawkq + (b & 1) * m.rawkq_stage, m.rawkq_stage / 2, kq_all + ((b + 2) % Cf::NKQ) * Cf::KQ, p.qkv_act, ptid, nt);
+    }
+    if (prep && prepares) {
+      float *gram1 = gram_all + (b1 & 1) * Cf::GJ * Cf::GR;
+      if constexpr (GATE == 1) {
+        if (slow)
+          block_gram_products<Cf>(kq1, reinterpret_cast<const float *>(smem + m.alpha + (b1 & 1) * m.alpha_stage), gram1, nv1, p.post, ptid, nt);
+        else
+          block_gram<Cf>(reinterpret_cast<const float *>(smem + m.kh), DK, Cf::KB, reinterpret_cast<const float *>(smem + m.kt) + (b1 & 1) * J * Cf::KT, Cf::KT,
+                         gram1, ptid, nt);
+      } else {
+        block_gram<Cf>(kq1, 2 * DK, 0, kq1, 0, gram1, ptid, nt);
+      }
+    }
+    if (holds && b >= 0) {
+      const int nvalid = min(C, p.T - b * C);
+      const float *vec = GATE == 1 ? reinterpret_cast<const float *>(smem + m.kt) + ((b & 1) * J + j) * Cf::KT : kq_all + (b % Cf::NKQ) * Cf::KQ;
+      const float *upd = GATE == 1 ? reinterpret_cast<const float *>(smem + m.kb) + ((b & 1) * J + j) * Cf::KB : vec;
+      constexpr int US = GATE == 1 ? DK : 2 * DK;
+      const float *gram = gram_all + ((b & 1) * Cf::GJ + (GATE == 1 ? j : 0)) * Cf::GR;
+      const unsigned char *gates = smem + m.gates + (b & 1) * m.gates_stage;
+      IO *ost = reinterpret_cast<IO *>(smem + m.ost) + warp * C * CPW;
+      float *cb = reinterpret_cast<float *>(smem + m.cbuf) + warp * Cf::CB;
+      float *xch = cb + lane * 2 * OC;
+      // an update coefficient goes to the lanes of its row as a pair of equal values, ready for the packed FMAs, and, when
+      // neighbouring registers of a lane may hold neighbouring columns in either order (OC = 1), in both orders
+      constexpr int TS = Cf::NCOPY * Cf::RW * 2;  // floats per token
+      const int rowb = (ln.cg * J + j) * NC;
+      float *cw = cb + (rowb + mask) * 2;
+      auto put = [&](int t, int o, float x) {
+        *reinterpret_cast<float2 *>(cw + t * TS + o * 2) = make_float2(x, x);
+        if constexpr (Cf::NCOPY == 2) *reinterpret_cast<float2 *>(cb + t * TS + (Cf::RW + rowb + (mask ^ 1)) * 2) = make_float2(x, x);
+      };
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        // state times k_t and q_t, reduced over the key slices.  The butterfly of token t-1 (val) runs between the FMAs of
+        // token t, a round after each operand load.  The loop stays rolled: straight-line code for all tokens is fetched
+        // slower than it is issued.
+        float val[2 * NC];
+#pragma unroll
+        for (int i = 0; i < 2 * NC; ++i) val[i] = 0.f;
+        auto round = [&](int n) {  // half of the columns to the partner
+          const int h = NC >> (n + 1), d = G >> (n + 1);
+          if (d >= 1) {
+#pragma unroll
+            for (int i = 0; i < NC / 2; ++i) {
+              if (i < h) {
+                val[i] += __shfl_xor_sync(0xffffffffu, val[i + h], d);
+                val[NC + i] += __shfl_xor_sync(0xffffffffu, val[NC + i + h], d);
+              }
+            }
+          }
+        };
+        auto keep = [&](int t) {
+          float *dst = xch + t * 64 * OC;
+          if constexpr (OC == 1) *reinterpret_cast<float2 *>(dst) = make_float2(val[0], val[NC]);
+          else *reinterpret_cast<float4 *>(dst) = make_float4(val[0], val[1], val[NC], val[NC + 1]);
+        };
+        const float *vl = vec + g * 4;
+        float4 x = *reinterpret_cast<const float4 *>(vl), y = *reinterpret_cast<const float4 *>(vl + DK);
+#pragma unroll 1
+        for (int t = 0; t < C; ++t) {
+          float2 acc[2 * NC];
+#pragma unroll
+          for (int n = 0; n < L / 4; ++n) {
+            // the next operands are on their way while these are used (past the last token: of the token itself again)
+            const float *nx = n + 1 < L / 4 ? vl + (n + 1) * G * 4 : vl + (t + 1 < C ? 2 * DK : 0);
+            const float4 xn = *reinterpret_cast<const float4 *>(nx), yn = *reinterpret_cast<const float4 *>(nx + DK);
+#pragma unroll
+            for (int i = 0; i < NC; ++i) acc[i] = n == 0 ? mul2(w[i][0], make_float2(x.x, x.y)) : fma2(w[i][2 * n], make_float2(x.x, x.y), acc[i]);
+#pragma unroll
+            for (int i = 0; i < NC; ++i) acc[NC + i] = n == 0 ? mul2(w[i][0], make_float2(y.x, y.y)) : fma2(w[i][2 * n], make_float2(y.x, y.y), acc[NC + i]);
+#pragma unroll
+            for (int i = 0; i < NC; ++i) acc[i] = fma2(w[i][2 * n + 1], make_float2(x.z, x.w), acc[i]);
+#pragma unroll
+            for (int i = 0; i < NC; ++i) acc[NC + i] = fma2(w[i][2 * n + 1], make_float2(y.z, y.w), acc[NC + i]);
+            round(n);
+            x = xn; y = yn;
+          }
+          vl += 2 * DK;
+          keep((t + C - 1) % C);  // (for t = 0 nothing yet: the last slot is written again below)
+#pragma unroll
+          for (int i = 0; i < 2 * NC; ++i) val[i] = acc[i].x + acc[i].y;
+        }
+#pragma unroll
+        for (int n = 0; n < L / 4; ++n) round(n);
+        keep(C - 1);
+        __syncwarp();
+        if (pass == 0) {
+          wait(2, b);
+          if (!block_tokens<Cf, false>(p, m, ln, xch, put, gates, gram, ost, cols, nvalid, colw + mask, tok0 + (size_t)b * C)) break;
+        } else {
+          block_tokens<Cf, true>(p, m, ln, xch, put, gates, gram, ost, cols, nvalid, colw + mask, tok0 + (size_t)b * C);
+        }
+        __syncwarp();
+      }
+      if constexpr (GATE == 2) {  // c_t times the row's later decays; the product of all of them decays the state
+        float sfx[OC];
+#pragma unroll
+        for (int o = 0; o < OC; ++o) sfx[o] = 1.f;
+#pragma unroll
+        for (int t = C - 1; t >= 0; --t) {
+          float a[OC];
+          if (row_alpha) {
+            block_ld<float, OC>(reinterpret_cast<const float *>(gates + m.g_ar) + (t * J + j) * (cols + 4) + ln.lc, a);
+          } else {
+#pragma unroll
+            for (int o = 0; o < OC; ++o) a[o] = t < nvalid ? __ldg(p.alpha + (tok0 + (size_t)b * C + t) * J + j) : 1.f;
+          }
+#pragma unroll
+          for (int o = 0; o < OC; ++o) {
+            put(t, o, cw[t * TS + o * 2] * sfx[o]);
+            if (t < nvalid) sfx[o] *= a[o];
+          }
+        }
+#pragma unroll
+        for (int o = 0; o < OC; ++o) put(C, o, sfx[o]);
+      }
+      __syncwarp();
+      // finished outputs: vectors of up to 16 bytes
+      {
+        constexpr int VB = CPW * Cf::ES < 16 ? CPW * Cf::ES : 16, VE = VB / Cf::ES, VPT = CPW / VE;
+        for (int e = lane; e < nvalid * VPT; e += 32) {
+          const int t = e / VPT, c = (e - t * VPT) * VE, col = col0 + warp * CPW + c;
+          if (col < p.Dv) {
+            IO *dst = (IO *)p.o + (tok0 + (size_t)b * C + t) * p.Dv + col;
+            const IO *src = ost + t * CPW + c;
+            if constexpr (VB == 16) *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
+            else if constexpr (VB == 8) *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(src);
+            else *reinterpret_cast<uint32_t *>(dst) = *reinterpret_cast<const uint32_t *>(src);
+          }
+        }
+      }
+      // ---- W <- (decays of the block) W + sum_t c_t k_t ----
+      const float *cr = cb + ((mask & 1) * Cf::RW + rowb) * 2;
+      auto coeff = [&](int t, float2(&c2)[NC]) {
+#pragma unroll
+        for (int i = 0; i < NC / 2; ++i) {
+          const float4 x = *reinterpret_cast<const float4 *>(cr + t * TS + (i ^ (mask >> 1)) * 4);
+          c2[2 * i] = make_float2(x.x, x.y);
+          c2[2 * i + 1] = make_float2(x.z, x.w);
+        }
+      };
+      if constexpr (GATE == 1) {
+        const float *ac = reinterpret_cast<const float *>(smem + m.ac) + ((b & 1) * J + j) * Cf::AC;
+#pragma unroll
+        for (int n = 0; n < L / 4; ++n) {
+          const float4 x = *reinterpret_cast<const float4 *>(ac + (n * G + g) * 4);
+#pragma unroll
+          for (int i = 0; i < NC; ++i) {
+            w[i][2 * n] = mul2(w[i][2 * n], make_float2(x.x, x.y));
+            w[i][2 * n + 1] = mul2(w[i][2 * n + 1], make_float2(x.z, x.w));
+          }
+        }
+      }
+      if constexpr (GATE == 2) {
+        float2 a2[NC];
+        coeff(C, a2);
+#pragma unroll
+        for (int i = 0; i < NC; ++i)
+#pragma unroll
+          for (int n = 0; n < L / 2; ++n) w[i][n] = mul2(w[i][n], a2[i]);
+      }
+      {
+        const float *ul = upd + g * 4;
+        float4 x = *reinterpret_cast<const float4 *>(ul);
+        float2 c2[NC];
+        coeff(0, c2);
+#pragma unroll 1
+        for (int t = 0; t < C; ++t) {
+          const int step = t + 1 < C ? 1 : 0;  // (past the last token: of the token itself again)
+          float2 cn[NC];
+#pragma unroll
+          for (int n = 0; n < L / 4; ++n) {
+            const float4 xn = *reinterpret_cast<const float4 *>(n + 1 < L / 4 ? ul + (n + 1) * G * 4 : ul + step * US);
+            if (n == 0) coeff(t + step, cn);
+#pragma unroll
+            for (int i = 0; i < NC; ++i) w[i][2 * n] = fma2(c2[i], make_float2(x.x, x.y), w[i][2 * n]);
+#pragma unroll
+            for (int i = 0; i < NC; ++i) w[i][2 * n + 1] = fma2(c2[i], make_float2(x.z, x.w), w[i][2 * n + 1]);
+            x = xn;
+          }
+#pragma unroll
+          for (int i = 0; i < NC; ++i) c2[i] = cn[i];
+          ul += US;
+        }
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---- registers -> state, carried distributions, statistics ----
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    const int col = colw + (i ^ mask);
+    if (p.W_out && holds && col < p.Dv) {
+      float *dst = p.W_out + (((size_t)bh * J + j) * p.Dv + col) * DK;
+#pragma unroll
+      for (int n = 0; n < L / 4; ++n)
+        __stcs(reinterpret_cast<float4 *>(dst + (n * G + g) * 4), make_float4(w[i][2 * n].x, w[i][2 * n].y, w[i][2 * n + 1].x, w[i][2 * n + 1].y));
+    }
+  }
+  if constexpr (Cf::EXT) {
+    constexpr float kLn2 = 0.6931471805599453f;
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      const int col = colw + mask + o;
+      const float hr = block_sum_j<Cf>(ln.s_rh[o]), hq = block_sum_j<Cf>(ln.s_qh[o]);
+      if (!holds || col >= p.Dv) continue;  // (uniform over the J lanes of a column; the shuffles are above)
+      const size_t at = ((size_t)bh * J + j) * p.Dv + col, ate = (size_t)bh * p.Dv + col;
+      if (temporal && p.r_out) p.r_out[at] = ln.rp[o];
+      if (temporal && p.rho_out) p.rho_out[at] = ln.rho[o];
+      // each element belongs to one lane of one block: plain read-modify-write
+      if (p.r_sum) p.r_sum[at] += ln.s_r[o];
+      if (p.rho_sum) p.rho_sum[at] += ln.s_q[o];
+      if (j == 0 && p.r_ent) p.r_ent[ate] -= hr * kLn2;
+      if (j == 0 && p.rho_ent) p.rho_ent[ate] -= hq * kLn2;
+    }
+  }
+}
+
+// ---- host-side launch of one instantiation -----------------------------------------------
+template <class Cf>
+bool block_make_maps(const ScanParams &p, int cols, BlockMaps *m) {
+  const cuuint64_t BH = (cuuint64_t)p.B * p.H, T = (cuuint64_t)p.T, Dv = (cuuint64_t)p.Dv, J = Cf::J, DK = Cf::DK, es = Cf::ES;
+  const CUtensorMapDataType io = es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  const CUtensorMapSwizzle none = CU_TENSOR_MAP_SWIZZLE_NONE;
+  auto rows = [&](CUtensorMap *map, const void *base, cuuint64_t width, int box_width) {  // [BH][T][width]
+    const cuuint64_t dims[3] = {width, T, BH}, strides[2] = {width * es, T * width * es};
+    const cuuint32_t box[3] = {(cuuint32_t)box_width, (cuuint32_t)Cf::C, 1};
+    return tma_encode(map, base, 3, dims, strides, box, none, io);
+  };
+  auto gates = [&](CUtensorMap *map, const void *base, cuuint64_t width, int box_width, cuuint64_t bytes, CUtensorMapDataType type) {  // [BH][T][J][width]
+    const cuuint64_t dims[4] = {width, J, T, BH}, strides[3] = {width * bytes, J * width * bytes, T * J * width * bytes};
+    const cuuint32_t box[4] = {(cuuint32_t)box_width, (cuuint32_t)J, (cuuint32_t)Cf::C, 1};
+    return tma_encode(map, base, 4, dims, strides, box, none, type);
+  };
+  bool ok = rows(&m->k, p.k, DK, Cf::DK) && rows(&m->q, p.q, DK, Cf::DK) && rows(&m->v, p.v, Dv, cols);
+  ok = ok && gates(&m->be, p.beta_logit, Dv, cols + Cf::PAD, es, io) && gates(&m->pk, p.pik_logit, Dv, cols + Cf::PAD, es, io) &&
+       gates(&m->pq, p.piq_logit, Dv, cols + Cf::PAD, es, io);
+  if (p.temporal) ok = ok && rows(&m->gk, p.gk_logit, Dv, cols) && rows(&m->gq, p.gq_logit, Dv, cols);
+  if (Cf::GATE == 1) ok = ok && gates(&m->al, p.alpha, DK, Cf::DK, 4, CU_TENSOR_MAP_DATA_TYPE_FLOAT32);
+  if (Cf::GATE == 2 && p.gran == SWILA_GATE_PER_OUT) ok = ok && gates(&m->al, p.alpha, Dv, cols + 4, 4, CU_TENSOR_MAP_DATA_TYPE_FLOAT32);
+  return ok;
+}
+
+// Warps (column slices of CPW) per thread block.  More warps share the operand preparation; fewer spread a small problem
+// over the SMs: halved while the grid would leave SMs without a block and the slice stays a multiple of 8 columns.
+template <class Cf>
+int block_warps(const ScanParams &p, int sms) {
+  const long long bh = (long long)p.B * p.H;
+  int nw = 1;
+  while (nw < 4 && nw * Cf::CPW < p.Dv && 2 * nw * Cf::CPW + Cf::PAD <= 256) nw *= 2;  // a copy box has at most 256 columns
+  while (nw > 1 && (nw / 2 * Cf::CPW) % 8 == 0 && bh * ((p.Dv + nw * Cf::CPW - 1) / (nw * Cf::CPW)) < sms) nw /= 2;
+  while ((nw * Cf::CPW) % 8 != 0) nw *= 2;
+  return nw;
+}
+
+template <class Cf>
+int launch_block(const LaunchArgs &a, int *err, int sms) {
+  const int nw = block_warps<Cf>(a.p, sms), cols = nw * Cf::CPW;
+  const BlockSmem m = block_smem<Cf>(nw, a.p.temporal != 0, Cf::GATE == 2 && a.p.gran == SWILA_GATE_PER_OUT);
+  const long long grid = (long long)a.p.B * a.p.H * ((a.p.Dv + cols - 1) / cols);
+  if (m.total > 227 * 1024) return -1000;
+  if (grid <= 0 || grid > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
+  // one block per SM anyway: four more warps take the preparation off the state warps
+  const int prep = grid <= sms ? 4 : 0;
+  BlockMaps maps;
+  if (!block_make_maps<Cf>(a.p, cols, &maps)) return (int)cudaErrorInvalidValue;
+  auto kern = swila_block_kernel<Cf>;
+  static std::atomic<uint64_t> granted;
+  cudaError_t e = allow_smem((const void *)kern, 227 * 1024, granted);  // (the size differs from launch to launch)
+  if (e != cudaSuccess) return (int)e;
+  kern<<<(unsigned)grid, (nw + prep) * 32, m.total, a.stream>>>(a.p, maps, nw, err);
+  return (int)cudaGetLastError();
+}
+
+}  // namespace swila

@@ -1,0 +1,46 @@
+// Instantiations of the blocked scan: one translation unit per (key dimension, decay mode), compiled with
+// -DSWILA_DK=<16|64|128> -DSWILA_GATE=<0|1|2>.
+#include "swila_block.cuh"
+
+#ifndef SWILA_DK
+#error "compile with -DSWILA_DK, -DSWILA_GATE"
+#endif
+
+namespace swila {
+
+namespace {
+template <typename IO, int J, bool EXT>
+int pick(const LaunchArgs &a, int *err, int sms) {
+  constexpr int DK = SWILA_DK, GATE = SWILA_GATE;
+  if constexpr (GATE == 1 && DK == 128 && J == 16) {
+    return -1000;  // the decayed operands of 16 components do not fit shared memory
+  } else {
+    // tokens per block: the decayed operands of many components at once leave room for four only
+    constexpr int C = (GATE == 1 && J * DK >= 1024) ? 4 : 8;
+    // columns per lane: 128 state registers, except where a lane would own more than two columns of the E-step
+    constexpr int NC = DK == 16 ? 2 : (J == 16 ? (DK == 64 ? 4 : 2) : (J == 8 && DK == 128 ? 4 : 8));
+    return launch_block<BlockCfg<IO, J, DK, NC, C, GATE, EXT>>(a, err, sms);
+  }
+}
+template <typename IO, bool EXT>
+int pick_j(const LaunchArgs &a, int *err, int sms) {
+  switch (a.J) {
+    case 1: return pick<IO, 1, EXT>(a, err, sms);
+    case 2: return pick<IO, 2, EXT>(a, err, sms);
+    case 4: return pick<IO, 4, EXT>(a, err, sms);
+    case 8: return pick<IO, 8, EXT>(a, err, sms);
+    case 16: return pick<IO, 16, EXT>(a, err, sms);
+    default: return -1000;
+  }
+}
+}  // namespace
+
+// Returns a cudaError_t value (>= 0), or -1000 when the combination is not compiled.
+template <>
+int block_dispatch<SWILA_DK, SWILA_GATE>(const LaunchArgs &a, int *err, int sms) {
+  const bool ext = a.p.temporal || a.p.r_debug || a.p.r_sum || a.p.r_ent || a.p.rho_sum || a.p.rho_ent;
+  if (a.io_dtype == SWILA_IO_BF16) return ext ? pick_j<__nv_bfloat16, true>(a, err, sms) : pick_j<__nv_bfloat16, false>(a, err, sms);
+  return ext ? pick_j<float, true>(a, err, sms) : pick_j<float, false>(a, err, sms);
+}
+
+}  // namespace swila

@@ -1,0 +1,974 @@
+// Register-tile kernel of the SwiLA recurrence (Sec. 3.2, Eqs. 3.3-3.5) for sm_100a: 16 tokens at a time, the state in the
+// accumulator fragments of warp-level matrix instructions, FP32-grade operands.
+//
+// Over a block of 16 tokens from state W0, for every row (component j, output column d), the same recurrence as the scan,
+// only the order of the additions differs:
+//
+//   p_t = W0.k_t, r_t = W0.q_t                                             (matrix instructions)
+//   token by token: delta = v - p_t, E-step, c_t; p_t' += c_t k_t.k_t'      (FP32 ALUs, one lane per row)
+//   r_t += sum_{s<=t} c_s k_s.q_t,  W += sum_t c_t k_t                      (matrix instructions)
+//   o_t = sum_j pi^q_j r_t                                                  (in the fragment layout)
+//
+// A warp owns R = 16 MT rows (R / J columns of all J components) with all Dk key dimensions: MT x Dk/8 accumulator tiles of
+// m16n8k16, 128 registers per lane.  An accumulator tile read as two-element rows is the A fragment of the next product,
+// so the state never leaves the registers: it is split into three bf16 parts (24 bits) where it is multiplied.  k and q in bf16 are exact B
+// operands; in fp32, or activated in the kernel, they are three parts as well and the six products above 2^-24 are formed.  A
+// warp needs no other warp for its rows: no hand-overs between roles, and two or more warps per scheduler fill each
+// other's gaps.
+//
+// Why warp-level instructions and not tcgen05: a block's products are 64 rows x 32 vectors x 64 key dimensions per warp, and
+// between any two of them stands the serial E-step.  With tcgen05 the state would live in tensor memory and cross it twice per
+// block in each direction (split into parts, written back), the E-step's rows would be tied to tensor-memory lanes, and roles would
+// meet on barriers: the chunked kernel, which is built that way, runs 128 rows per SM at ~8,400 cycles per 32 tokens, bound
+// by those crossings and by one warp's chain per scheduler.  m16n8k16 takes 8 cycles per scheduler, measured.
+#pragma once
+
+#include "swila_common.cuh"
+#include "swila_tma_maps.h"
+#include "swila_umma.cuh"
+
+namespace swila {
+
+template <typename IO_, int J_, int DK_, int MT_, bool EXT_, int NPK_>
+struct TileCfg {
+  using IO = IO_;
+  static constexpr int J = J_, DK = DK_, MT = MT_, NPK = NPK_;
+  static constexpr bool EXT = EXT_;  // the instantiation with the Temporal priors, r_debug and the statistics
+  static constexpr int C = 16;       // tokens per block: the K extent of one matrix instruction
+  static constexpr int ES = (int)sizeof(IO);
+  // bf16 parts of the state where it is multiplied, and products kept of the readouts' corrections (parts i, j with i + j below it): with
+  // exact bf16 k and q what the chunked kernel has (16 bits of the state and of the corrections, 24 of what is added to the
+  // state); else everything at 24 bits
+  static constexpr int NPW = NPK == 1 ? 2 : 3, RPARTS = NPK == 1 ? 2 : 3;
+  static constexpr int KS = DK / 16, N8 = DK / 8;  // K steps of the products with the state; its accumulator tiles per 16 rows
+  static constexpr int R = 16 * MT, CPW = R / J;   // rows and columns per warp; row = component * CPW + column
+  // E-step: RL rows per lane, CL components of OCL columns; LPC lanes share a column.  lane = part * LCOLS + column slot
+  static constexpr int RL = R / 32, CL = J < RL ? J : RL, OCL = RL / CL, LPC = J / CL, LCOLS = 32 / LPC;
+  // fragment layout (rows g and g + 8 of each tile, g = lane / 4): column slots per lane and components in the lane per slot
+  static constexpr int NCS = CPW >= 8 ? CPW / 8 : 1, NCL = 2 * MT / NCS, GC = CPW >= 8 ? 8 : CPW;  // GC: columns among the 8 values of g
+  static_assert(R % 32 == 0 && J * CPW == R && CL * OCL == RL && LPC * CL == J, "row split");
+  static constexpr int PAD = 16 / ES;
+  static constexpr int NB = 3;                                        // ring of operand tiles
+  static constexpr int PART = (DK / 64) * 32 * 128;                   // one part of [k ; q] of a block: rows of 128 bytes, 128-byte swizzle
+  static constexpr int RAWKQ = NPK == 1 ? 0 : 2 * C * DK * ES;        // k and q as they arrive, when they have to be converted
+  static constexpr int GK = C * 20 * 4;                               // k_s.k_t, fp32 rows of 20
+  static constexpr int GQP = C * 48;                                  // one part of k_s.q_t (s <= t) as [t][s] bf16, rows of 48 bytes
+  // exchange rows of a warp, 7 units of 16 bytes (an odd number: the rows of a matrix load fall into different banks).  First
+  // p_0 .. p_15 in units 0..3; then the coefficients' parts, of tokens 0..7 in units 0, 1, 4, of tokens 8..15 in units 2, 3, 5; then
+  // the outputs.
+  static constexpr int XROW = 112, XCH = R * XROW;
+  static_assert(XCH >= C * CPW * ES, "the outputs take the place of the coefficients");
+  static constexpr int WROW = 20, WB = EXT ? R * WROW * 4 : 0;        // readout weights (Temporal): floats per row
+};
+
+__host__ __device__ constexpr int tile_up128(int n) { return (n + 127) & ~127; }
+
+struct TileSmem {
+  int kq, rawkq, gates, gates_stage, g_be, g_pk, g_pq, g_gk, g_gq, gk, gq, xch, wb, bars, total;
+};
+template <class Cf>
+__host__ __device__ inline TileSmem tile_smem(int nwarps, bool temporal, int gate_bufs) {
+  TileSmem m;
+  const int cols = nwarps * Cf::CPW, grow = cols + Cf::PAD;
+  const int gate = tile_up128(Cf::C * Cf::J * grow * Cf::ES), vec = tile_up128(Cf::C * cols * Cf::ES);
+  int off = 0;
+  m.kq = off; off += Cf::NB * Cf::NPK * Cf::PART;
+  m.rawkq = off; off += 2 * Cf::RAWKQ;
+  m.gates = off;
+  m.g_be = vec; m.g_pk = m.g_be + gate; m.g_pq = m.g_pk + gate; m.g_gk = m.g_pq + gate;
+  m.g_gq = m.g_gk + (temporal ? vec : 0); m.gates_stage = m.g_gq + (temporal ? vec : 0);
+  off += gate_bufs * m.gates_stage;
+  m.gk = off; off += 2 * Cf::GK;
+  m.gq = off; off += 2 * 3 * Cf::GQP;
+  m.xch = off; off += nwarps * Cf::XCH;
+  m.wb = off; off += temporal ? nwarps * Cf::WB : 0;
+  m.bars = off; off += 64;
+  m.total = off + 1024;  // the kernel aligns its window to 1024 bytes (the swizzle is a function of the address)
+  return m;
+}
+
+struct TileMaps {
+  CUtensorMap k, q, v, be, pk, pq, gk, gq;
+};
+
+// ---- instructions ----------------------------------------------------------------------------
+__device__ __forceinline__ void tile_mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void tile_ldsm(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void tile_ldsm_t(uint32_t (&r)[4], uint32_t addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+// x = part 0 + part 1 (+ part 2), 8 bits each; two values packed per part
+template <int N>
+__device__ __forceinline__ void tile_split(float x0, float x1, uint32_t (&p)[N]) {
+  float2 x = make_float2(x0, x1);
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x.x, x.y);
+    p[n] = *reinterpret_cast<const uint32_t *>(&h);
+    if (n + 1 < N) x = __fadd2_rn(x, make_float2(-__uint_as_float(p[n] << 16), -__uint_as_float(p[n] & 0xffff0000u)));
+  }
+}
+// Byte offset of a 16-byte unit (8 key dimensions) of a vector in one part of an operand tile (what a tensor copy with the
+// 128-byte swizzle writes): vectors 0..15 are k, 16..31 are q.
+__device__ __forceinline__ int tile_at(int row, int unit) { return (unit >> 3) * 4096 + row * 128 + (((unit & 7) ^ (row & 7)) << 4); }
+
+// Byte offset, in an exchange row, of one part of the coefficients of tokens 0..7 (half 0) or 8..15.
+__host__ __device__ constexpr int tile_c_at(int part, int half) { return part < 2 ? (2 * half + part) * 16 : (4 + half) * 16; }
+// Loads that stay where they are written: the serial part is unrolled over its 16 tokens, and a compiler that is free to fetch
+// all their gates first has no registers left for the state.
+__device__ __forceinline__ float tile_lds(uint32_t addr, const float *) {
+  float x;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x) : "r"(addr));
+  return x;
+}
+__device__ __forceinline__ float tile_lds(uint32_t addr, const __nv_bfloat16 *) {
+  unsigned short x;
+  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(x) : "r"(addr));
+  return __uint_as_float((uint32_t)x << 16);
+}
+__device__ __forceinline__ float4 tile_lds4(uint32_t addr) {
+  float4 x;
+  asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(addr));
+  return x;
+}
+
+// Bounded wait (two seconds of wall time); on expiry the error word is set and every later wait of the thread is skipped.
+static __device__ __noinline__ bool tile_wait_poll(uint64_t *bar, uint32_t parity, int *err) {
+  const unsigned long long t0 = umma::global_timer_ns();
+#pragma unroll 1
+  for (uint32_t i = 1;; ++i) {
+    if (umma::mbar_try_wait(bar, parity)) return true;
+    if ((i & 255u) == 0 && umma::global_timer_ns() - t0 > 2000000000ull) {
+      atomicCAS(err, 0, (int)(((threadIdx.x >> 5) + 1) * 65536 + (umma::smem_u32(bar) & 0xffffu)));
+      return false;
+    }
+  }
+}
+
+// ---- preparation -----------------------------------------------------------------------------
+// k and q of one block into the three parts of an operand tile; with `act` after SiLU and the L2 norm over the key
+// dimension (App. B.2, App. D.1): the DK / 8 work items of a vector are adjacent lanes of one warp.
+template <class Cf>
+__device__ __forceinline__ void tile_convert(const unsigned char *raw, unsigned char *tile, bool act, int tid, int nt) {
+  using IO = typename Cf::IO;
+  constexpr int DK = Cf::DK, UPV = DK / 8;
+  for (int i = tid; i < 32 * UPV; i += nt) {
+    const int vec = i / UPV, u = i - vec * UPV;
+    const IO *src = reinterpret_cast<const IO *>(raw) + vec * DK + u * 8;
+    float x[8];
+    if constexpr (sizeof(IO) == 2) {
+      const uint4 y = *reinterpret_cast<const uint4 *>(src);
+      const uint32_t w[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int n = 0; n < 4; ++n) { x[2 * n] = __uint_as_float(w[n] << 16); x[2 * n + 1] = __uint_as_float(w[n] & 0xffff0000u); }
+    } else {
+      const float4 a = reinterpret_cast<const float4 *>(src)[0], b = reinterpret_cast<const float4 *>(src)[1];
+      x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+    }
+    if (act) {
+      float ss = 0.f;
+#pragma unroll
+      for (int n = 0; n < 8; ++n) { x[n] = silu_approx(x[n]); ss = fmaf(x[n], x[n], ss); }
+#pragma unroll
+      for (int off = 1; off < UPV; off <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+      const float inv = rsqrtf(ss + kL2Eps);
+#pragma unroll
+      for (int n = 0; n < 8; ++n) x[n] *= inv;
+    }
+    uint32_t p[4][3];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) tile_split(x[2 * n], x[2 * n + 1], p[n]);
+#pragma unroll
+    for (int s = 0; s < 3; ++s)
+      *reinterpret_cast<uint4 *>(tile + s * Cf::PART + tile_at(vec, u)) = make_uint4(p[0][s], p[1][s], p[2][s], p[3][s]);
+  }
+}
+
+// Half of a Gram matrix of a block (8 of its 16 columns, n8) by one warp.  which = 0: k_s.k_t as fp32 rows [s][t] for the E-step; 1: k_s.q_t, zero for s > t, as
+// [t][s] in three bf16 parts, the B operand of the readouts.
+template <class Cf>
+__device__ __forceinline__ void tile_gram(const unsigned char *tile, int which, int n8, float *gk, unsigned char *gq, int lane) {
+  float d[4] = {0.f, 0.f, 0.f, 0.f};
+  const uint32_t base = umma::smem_u32(tile);
+  const int arow = (which ? 16 : 0) + (lane & 7) + ((lane >> 3) & 1) * 8, brow = n8 * 8 + (lane & 7);
+  uint32_t b[Cf::NPK][4];  // (a matrix load of B brings two K steps)
+#pragma unroll
+  for (int ks = 0; ks < Cf::KS; ++ks) {
+    uint32_t a[Cf::NPK][4];
+#pragma unroll
+    for (int p = 0; p < Cf::NPK; ++p) {
+      tile_ldsm(a[p], base + p * Cf::PART + tile_at(arow, 2 * ks + (lane >> 4)));
+      if ((ks & 1) == 0) tile_ldsm(b[p], base + p * Cf::PART + tile_at(brow, 2 * ks + (lane >> 3)));
+    }
+#pragma unroll
+    for (int pa = 0; pa < Cf::NPK; ++pa)
+#pragma unroll
+      for (int pb = 0; pb < Cf::NPK; ++pb)
+        if (pa + pb < 3) {
+          tile_mma(d, a[pa], b[pb][(ks & 1) * 2], b[pb][(ks & 1) * 2 + 1]);
+        }
+  }
+  const int g = lane >> 2, t2 = (lane & 3) * 2;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int row = g + 8 * h, c = 8 * n8 + t2;
+    if (which == 0) {
+      *reinterpret_cast<float2 *>(gk + row * 20 + c) = make_float2(d[2 * h], d[2 * h + 1]);
+    } else {
+      uint32_t p[Cf::RPARTS];
+      tile_split(c <= row ? d[2 * h] : 0.f, c + 1 <= row ? d[2 * h + 1] : 0.f, p);
+#pragma unroll
+      for (int s = 0; s < Cf::RPARTS; ++s) *reinterpret_cast<uint32_t *>(gq + s * Cf::GQP + row * 48 + c * 2) = p[s];
+    }
+  }
+}
+
+// ---- the serial part of a block: RL rows per lane ------------------------------------------------
+template <class Cf>
+struct TileLane {
+  int comp0, col;  // first component; first column inside the warp's columns
+  float rp[Cf::RL], rho[Cf::RL];                                       // Temporal: carried distributions
+  float s_r[Cf::RL], s_rh[Cf::RL], s_q[Cf::RL], s_qh[Cf::RL];          // statistics (entropies in bits)
+};
+
+// Over the J components of a column: CL of them in the lane, the rest LCOLS lanes apart.
+// `shadow` is run once, behind the first shuffles.
+struct TileNothing { __device__ __forceinline__ void operator()() const {} };
+template <class Cf, class Op, class Shadow = TileNothing>
+__device__ __forceinline__ float tile_over_j(float x, Op op, Shadow shadow = Shadow()) {
+  constexpr int D = Cf::LCOLS;
+  if constexpr (Cf::LPC == 4) {  // three independent shuffles: shorter than two dependent rounds
+    const float a = __shfl_xor_sync(0xffffffffu, x, D), b = __shfl_xor_sync(0xffffffffu, x, 2 * D), c = __shfl_xor_sync(0xffffffffu, x, 3 * D);
+    shadow();
+    return op(op(x, a), op(b, c));
+  } else {
+#pragma unroll
+    for (int off = 1; off < Cf::LPC; off <<= 1) {
+      const float y = __shfl_xor_sync(0xffffffffu, x, off * D);
+      if (off == 1) shadow();
+      x = op(x, y);
+    }
+    if (Cf::LPC == 1) shadow();
+    return x;
+  }
+}
+struct TileAdd { __device__ __forceinline__ float operator()(float a, float b) const { return a + b; } };
+struct TileMax { __device__ __forceinline__ float operator()(float a, float b) const { return fmaxf(a, b); } };
+
+// The gates of a lane, one token ahead: raw, then activated.
+template <class Cf>
+struct TileGates {
+  uint32_t av, ag, at_gk;  // shared-memory addresses of the next token to be fetched: v, the gates of the lane's first row, the Temporal gate
+  int sv, sg;              // bytes from token to token
+  float v_raw[Cf::OCL], b_raw[Cf::RL], k_raw[Cf::RL], g_raw[Cf::OCL];
+  float v[Cf::OCL], b[Cf::RL], k[Cf::RL], g[Cf::OCL];
+
+  __device__ __forceinline__ void fetch(const TileSmem &m, int grow, bool temporal) {
+    const typename Cf::IO *const io = nullptr;  // (a type tag)
+#pragma unroll
+    for (int o = 0; o < Cf::OCL; ++o) {
+      v_raw[o] = tile_lds(av + o * Cf::LCOLS * Cf::ES, io);
+      if constexpr (Cf::EXT) g_raw[o] = temporal ? tile_lds(at_gk + o * Cf::LCOLS * Cf::ES, io) : 0.f;
+#pragma unroll
+      for (int c = 0; c < Cf::CL; ++c) {
+        const uint32_t at = ag + (c * grow + o * Cf::LCOLS) * Cf::ES;
+        b_raw[o * Cf::CL + c] = tile_lds(at + m.g_be, io);
+        k_raw[o * Cf::CL + c] = tile_lds(at + m.g_pk, io);
+      }
+    }
+    av += sv; ag += sg;
+    if constexpr (Cf::EXT) at_gk += sv;
+  }
+  __device__ __forceinline__ void activate(bool valid, bool act, bool temporal) {
+#pragma unroll
+    for (int o = 0; o < Cf::OCL; ++o) {
+      v[o] = Cf::NPK == 3 && act ? silu_approx(v_raw[o]) : v_raw[o];
+#pragma unroll
+      for (int c = 0; c < Cf::CL; ++c) {
+        const int r = o * Cf::CL + c;
+        b[r] = sigmoid_approx(b_raw[r]);
+        if (!valid) b[r] = 0.f;  // past the end of the sequence: no update
+        k[r] = k_raw[r] * kLog2e;
+      }
+      if (Cf::EXT && temporal) {  // the key-side prior enters a convex combination: normalised over the components (App. B.3)
+        g[o] = sigmoid_approx(g_raw[o]);
+        float mx = k[o * Cf::CL];
+#pragma unroll
+        for (int c = 1; c < Cf::CL; ++c) mx = fmaxf(mx, k[o * Cf::CL + c]);
+        mx = tile_over_j<Cf>(mx, TileMax());
+        float se = 0.f;
+#pragma unroll
+        for (int c = 0; c < Cf::CL; ++c) { k[o * Cf::CL + c] = ex2_approx(k[o * Cf::CL + c] - mx); se += k[o * Cf::CL + c]; }
+        const float ise = rcp_approx(tile_over_j<Cf>(se, TileAdd()));
+#pragma unroll
+        for (int c = 0; c < Cf::CL; ++c) k[o * Cf::CL + c] *= ise;
+      }
+    }
+  }
+  // the gates of token t ready, those of t + 1 on their way
+  __device__ __forceinline__ void prime(const ScanParams &p, const TileSmem &m, const TileLane<Cf> &ln, uint32_t gates, int cols, int wcol, int t, int nvalid) {
+    const int grow = cols + Cf::PAD, lc = wcol + ln.col;
+    const bool temporal = Cf::EXT && p.temporal != 0;
+    sv = cols * Cf::ES; sg = Cf::J * grow * Cf::ES;
+    av = gates + lc * Cf::ES + t * sv;
+    ag = gates + (ln.comp0 * grow + lc) * Cf::ES + t * sg;
+    if constexpr (Cf::EXT) at_gk = av + m.g_gk;
+    fetch(m, grow, temporal);
+    activate(t < nvalid, p.qkv_act, temporal);
+    fetch(m, grow, temporal);
+  }
+};
+
+// Eight tokens, tg .. tg + 7: slots 0..7 of the window P2 (pairs) hold their predictions and are left with their update coefficients,
+// slots 8..15 are the predictions of the eight after them (past the end of the block: dead).  EXACT subtracts the maximum before the
+// exponentials; without it the trip returns whether a normaliser of this lane left the safe range.
+//
+// What bounds it: the serial chain of a token (two exponential-unit instructions, one round of shuffles, ~110 cycles), and
+// with two rows per lane its instructions.  The loads are placed by hand, under the latency of the shuffles: free to move them, the
+// compiler fetched the gates of all tokens first and spilled the state (250 cycles per token, 139 as it is).
+template <class Cf, bool EXACT>
+__device__ __forceinline__ bool tile_trip(const ScanParams &p, const TileSmem &m, TileLane<Cf> &ln, TileGates<Cf> &gt, float2 (&P2)[Cf::RL][Cf::C / 2], uint32_t gk_s,
+                                          int grow, int tg, int nvalid, int col0, size_t tok) {
+  constexpr int J = Cf::J, C = Cf::C, RL = Cf::RL, CL = Cf::CL, OCL = Cf::OCL, GT = 8;
+  const bool temporal = Cf::EXT && p.temporal != 0;
+  auto P = [&](int r, int i) -> float & { return (i & 1) ? P2[r][i >> 1].y : P2[r][i >> 1].x; };
+  bool bad = false;
+  gk_s += tg * 84;  // row tg, column tg
+  float gk[C];      // k_t.k_t' of one token t with the slots of the window
+  auto push = [&](int i) {  // token tg + i into the slots from i + 2 on
+#pragma unroll
+    for (int r = 0; r < RL; ++r) {
+      const float cp = P(r, i);
+      const float2 c2 = make_float2(cp, cp);
+      if (i & 1) P(r, i + 2) = fmaf(cp, gk[i + 2], P(r, i + 2));
+#pragma unroll
+      for (int u = (i + 3) / 2; u < C / 2; ++u) P2[r][u] = fma2(c2, make_float2(gk[2 * u], gk[2 * u + 1]), P2[r][u]);
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < GT; ++i) {
+    const int t = tg + i;
+    float e[RL], x[RL], bd[RL];
+#pragma unroll
+    for (int o = 0; o < OCL; ++o) {
+#pragma unroll
+      for (int c = 0; c < CL; ++c) {
+        const int r = o * CL + c;
+        const float lk = temporal ? lg2_approx(fmaf(gt.g[o], gt.k[r] - ln.rp[r], ln.rp[r])) : gt.k[r];  // log of (1 - g) r_{t-1} + g pi^k
+        const float delta = gt.v[o] - P(r, i);
+        x[r] = fmaf(-kHalfLog2e * delta, delta, lk);
+        bd[r] = gt.b[r] * delta;
+      }
+      if constexpr (EXACT) {
+        float mx = x[o * CL];
+#pragma unroll
+        for (int c = 1; c < CL; ++c) mx = fmaxf(mx, x[o * CL + c]);
+        mx = tile_over_j<Cf>(mx, TileMax());
+#pragma unroll
+        for (int c = 0; c < CL; ++c) x[o * CL + c] -= mx;
+      }
+      float sum = 0.f;
+#pragma unroll
+      for (int c = 0; c < CL; ++c) { e[o * CL + c] = ex2_approx(x[o * CL + c]); sum += e[o * CL + c]; }
+      // Under the latency of the sum's shuffles: the previous token's pushes (only its push into this token stood on the serial
+      // chain), this token's products with the later ones, the next token's gates.
+      auto shadow = [&]() {
+        if (o + 1 < OCL) return;
+        if (i > 0) push(i - 1);
+#pragma unroll
+        for (int q = (i + 1) / 4; q < C / 4; ++q) {
+          const float4 y = tile_lds4(gk_s + i * 80 + q * 16);
+          gk[4 * q] = y.x; gk[4 * q + 1] = y.y; gk[4 * q + 2] = y.z; gk[4 * q + 3] = y.w;
+        }
+        gt.activate(t + 1 < nvalid, p.qkv_act, temporal);
+        gt.fetch(m, grow, temporal);  // (two tokens past the block at its end: inside shared memory, unused)
+      };
+      sum = tile_over_j<Cf>(sum, TileAdd(), shadow);
+      if constexpr (!EXACT) bad = bad || !(sum > 1e-30f && sum < 1e30f);
+      const float rs = rcp_approx(sum);
+#pragma unroll
+      for (int c = 0; c < CL; ++c) {
+        const int r = o * CL + c;
+        if constexpr (Cf::EXT) {
+          const float rr = e[r] * rs;
+          if (t < nvalid) {
+            ln.rp[r] = rr;
+            ln.s_r[r] += rr;
+            if (rr > 0.f) ln.s_rh[r] = fmaf(rr, lg2_approx(e[r]) - lg2_approx(sum), ln.s_rh[r]);
+            const int col = col0 + o * Cf::LCOLS;
+            if (p.r_debug && col < p.Dv) p.r_debug[((tok + t) * J + ln.comp0 + c) * p.Dv + col] = rr;
+          }
+        }
+        P(r, i) = (bd[r] * e[r]) * rs;  // the update coefficient beta r delta
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < RL; ++r) P(r, i + 1) = fmaf(P(r, i), gk[i + 1], P(r, i + 1));  // the push that the next token waits for
+  }
+  push(GT - 1);
+  return bad;
+}
+
+// The exact trip on memory, out of line: rare, and its registers are not the fast path's.  The trip's predictions are in the exchange
+// rows (units tg / 4 and on, of the whole block); coefficients and later predictions are left there.
+template <class Cf>
+__device__ __noinline__ void tile_trip_again(const ScanParams *p, const TileSmem *m, unsigned char *xch, uint32_t gates, uint32_t gk_s, int cols, int wcol, int tg, int nvalid,
+                                             int col0, size_t tok) {
+  const int lane = threadIdx.x & 31;
+  TileLane<Cf> ln;
+  ln.comp0 = (lane / Cf::LCOLS) * Cf::CL;
+  ln.col = lane % Cf::LCOLS;
+#pragma unroll
+  for (int i = 0; i < Cf::RL; ++i) ln.rp[i] = ln.rho[i] = ln.s_r[i] = ln.s_rh[i] = ln.s_q[i] = ln.s_qh[i] = 0.f;
+  float2 P2[Cf::RL][Cf::C / 2];
+  auto row = [&](int i) { return reinterpret_cast<float2 *>(xch + ((ln.comp0 + i % Cf::CL) * Cf::CPW + ln.col + (i / Cf::CL) * Cf::LCOLS) * Cf::XROW + tg * 4); };
+  const int slots = tg == 0 ? Cf::C : 8;
+#pragma unroll
+  for (int i = 0; i < Cf::RL; ++i)
+#pragma unroll
+    for (int u = 0; u < Cf::C / 2; ++u) P2[i][u] = 2 * u < slots ? row(i)[u] : make_float2(0.f, 0.f);
+  TileGates<Cf> gt;
+  gt.prime(*p, *m, ln, gates, cols, wcol, tg, nvalid);
+  tile_trip<Cf, true>(*p, *m, ln, gt, P2, gk_s, cols + Cf::PAD, tg, nvalid, col0, tok);
+#pragma unroll
+  for (int i = 0; i < Cf::RL; ++i)
+#pragma unroll
+    for (int u = 0; u < Cf::C / 2; ++u)
+      if (2 * u < slots) row(i)[u] = P2[i][u];
+}
+
+// Temporal / statistics: the readout weights of a block, row by row (Temporal: to wb, [row][WROW]).
+template <class Cf>
+__device__ __forceinline__ void tile_weights(const ScanParams &p, const TileSmem &m, TileLane<Cf> &ln, const unsigned char *gates, float *wb, int cols, int wcol, int nvalid) {
+  using IO = typename Cf::IO;
+  constexpr int J = Cf::J, C = Cf::C, CL = Cf::CL;
+  const int grow = cols + Cf::PAD, lc = wcol + ln.col;
+  const bool temporal = p.temporal != 0, stats = p.rho_sum || p.rho_ent;
+  if (!temporal && !stats) return;
+  const IO *gpq = reinterpret_cast<const IO *>(gates + m.g_pq) + ln.comp0 * grow + lc;
+  const IO *ggq = reinterpret_cast<const IO *>(gates + m.g_gq) + lc;
+#pragma unroll 1
+  for (int t = 0; t < C; ++t) {
+#pragma unroll
+    for (int o = 0; o < Cf::OCL; ++o) {
+      float e[CL], mx = -3.0e38f, se = 0.f;
+#pragma unroll
+      for (int c = 0; c < CL; ++c) { e[c] = to_f32(gpq[t * J * grow + c * grow + o * Cf::LCOLS]) * kLog2e; mx = fmaxf(mx, e[c]); }
+      mx = tile_over_j<Cf>(mx, TileMax());
+#pragma unroll
+      for (int c = 0; c < CL; ++c) { e[c] = ex2_approx(e[c] - mx); se += e[c]; }
+      const float ise = rcp_approx(tile_over_j<Cf>(se, TileAdd()));
+      const float g = temporal ? sigmoid_approx(to_f32(ggq[t * cols + o * Cf::LCOLS])) : 0.f;
+#pragma unroll
+      for (int c = 0; c < CL; ++c) {
+        const int r = o * CL + c;
+        float w = e[c] * ise;
+        if (temporal) {
+          if (t < nvalid) ln.rho[r] = fmaf(g, w - ln.rho[r], ln.rho[r]);  // (1 - g) rhobar_{t-1} + g pi^q
+          w = ln.rho[r];
+          wb[((ln.comp0 + c) * Cf::CPW + ln.col + o * Cf::LCOLS) * Cf::WROW + t] = w;
+        }
+        if (stats && t < nvalid) {
+          ln.s_q[r] += w;
+          if (w > 0.f) ln.s_qh[r] = fmaf(w, lg2_approx(w), ln.s_qh[r]);
+        }
+      }
+    }
+  }
+}
+
+// ---- the kernel ---------------------------------------------------------------------------
+template <class Cf>
+__global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
+    swila_tile_kernel(const __grid_constant__ ScanParams p, const __grid_constant__ TileMaps maps, const int nwarps, const int gate_bufs, int *err) {
+  using IO = typename Cf::IO;
+  using namespace umma;
+  constexpr int J = Cf::J, DK = Cf::DK, C = Cf::C, MT = Cf::MT, KS = Cf::KS, N8 = Cf::N8, CPW = Cf::CPW, RL = Cf::RL, NPK = Cf::NPK;
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // `nwarps` warps hold the state; warps beyond them, if any, prepare the operands (else the state warps do)
+  const int pw0 = (int)(blockDim.x >> 5) > nwarps ? nwarps : 0;
+  const bool holds = warp < nwarps, prepares = warp >= pw0;
+  const int ptid = tid - pw0 * 32, nt = blockDim.x - pw0 * 32;
+  const int cols = nwarps * CPW;
+  const bool temporal = Cf::EXT && p.temporal != 0;
+  const TileSmem m = tile_smem<Cf>(nwarps, temporal, gate_bufs);
+  const int nslice = (p.Dv + cols - 1) / cols;
+  const int bh = blockIdx.x / nslice, col0 = (blockIdx.x - bh * nslice) * cols;
+  const size_t tok0 = (size_t)bh * p.T;
+  const int nb = (p.T + C - 1) / C;
+  uint64_t *bars = reinterpret_cast<uint64_t *>(smem + m.bars);  // k, q [3]; gates [2]
+
+  const int g = lane >> 2, t2 = (lane & 3) * 2;
+  TileLane<Cf> ln;
+  ln.comp0 = (lane / Cf::LCOLS) * Cf::CL;
+  ln.col = lane % Cf::LCOLS;
+  const int wcol = warp * CPW;  // the warp's first column inside the slice
+#pragma unroll
+  for (int r = 0; r < RL; ++r) {
+    ln.rp[r] = ln.rho[r] = 1.0f / J;
+    ln.s_r[r] = ln.s_rh[r] = ln.s_q[r] = ln.s_qh[r] = 0.f;
+    const int col = col0 + wcol + ln.col + (r / Cf::CL) * Cf::LCOLS;
+    if (temporal && holds && col < p.Dv) {
+      const size_t at = ((size_t)bh * J + ln.comp0 + r % Cf::CL) * p.Dv + col;
+      if (p.r_in) ln.rp[r] = p.r_in[at];
+      if (p.rho_in) ln.rho[r] = p.rho_in[at];
+    }
+  }
+
+  if (tid == 0) {
+    for (int i = 0; i < 3; ++i) mbar_init(&bars[i], 1);
+    for (int i = 3; i < 5; ++i) mbar_init(&bars[i], nt >= 128 ? 4 : 1);  // the threads that issue the gates' copies
+    mbar_fence_init();
+  }
+  __syncthreads();
+  // tensor copies of block b; the buffers were last read through ordinary loads, hence the proxy fence
+  auto load_kq = [&](int b) {
+    uint64_t *bar = &bars[NPK == 1 ? b % 3 : b & 1];
+    mbar_arrive_expect_tx(bar, 2 * C * DK * Cf::ES);
+    if constexpr (NPK == 1) {
+      unsigned char *dst = smem + m.kq + (b % Cf::NB) * Cf::PART;
+#pragma unroll
+      for (int hf = 0; hf < DK / 64; ++hf) {
+        tma_load_3d(dst + hf * 4096, &maps.k, hf * 64, b * C, bh, bar);
+        tma_load_3d(dst + hf * 4096 + 2048, &maps.q, hf * 64, b * C, bh, bar);
+      }
+    } else {
+      unsigned char *dst = smem + m.rawkq + (b & 1) * Cf::RAWKQ;
+      tma_load_3d(dst, &maps.k, 0, b * C, bh, bar);
+      tma_load_3d(dst + Cf::RAWKQ / 2, &maps.q, 0, b * C, bh, bar);
+    }
+  };
+  // the gates' copies in up to four parts, issued by as many warps: one thread takes several hundred cycles for all of them
+  auto load_gates = [&](int b, int part, int parts) {
+    unsigned char *dst = smem + m.gates + (gate_bufs == 2 ? b & 1 : 0) * m.gates_stage;
+    uint64_t *bar = &bars[3 + (b & 1)];
+    const int vec = C * cols * Cf::ES, gate = C * J * (cols + Cf::PAD) * Cf::ES;
+    const bool mine[4] = {part == 0, part == 1 % parts, part == 2 % parts, part == 3 % parts};
+    mbar_arrive_expect_tx(bar, (mine[0] ? vec * (temporal ? 3 : 1) : 0) + ((int)mine[1] + mine[2] + mine[3]) * gate);
+    if (mine[0]) {
+      tma_load_3d(dst, &maps.v, col0, b * C, bh, bar);
+      if (temporal) {
+        tma_load_3d(dst + m.g_gk, &maps.gk, col0, b * C, bh, bar);
+        tma_load_3d(dst + m.g_gq, &maps.gq, col0, b * C, bh, bar);
+      }
+    }
+    if (mine[1]) tma_load_4d(dst + m.g_be, &maps.be, col0, 0, b * C, bh, bar);
+    if (mine[2]) tma_load_4d(dst + m.g_pk, &maps.pk, col0, 0, b * C, bh, bar);
+    if (mine[3]) tma_load_4d(dst + m.g_pq, &maps.pq, col0, 0, b * C, bh, bar);
+  };
+  bool failed = false;
+  auto wait = [&](int bar_index, int parity) {
+    uint64_t *bar = &bars[bar_index];
+    if (!failed && !mbar_try_wait(bar, parity) && !tile_wait_poll(bar, parity, err)) failed = true;
+  };
+  auto wait_kq = [&](int b) {
+    if constexpr (NPK == 1) wait(b % 3, (b / 3) & 1);
+    else wait(b & 1, (b >> 1) & 1);
+  };
+  if (ptid == 0) load_kq(0);
+
+  // ---- state -> accumulator tiles: tile (mt, n8), rows g and g + 8 of its 16, key dims 8 n8 + t2 + {0, 1} ----
+  float w[MT][N8][4];
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int rho = mt * 16 + h * 8 + g, comp = rho / CPW, col = col0 + wcol + rho % CPW;
+      const float *src = (p.W_in && holds && col < p.Dv) ? p.W_in + (((size_t)bh * J + comp) * p.Dv + col) * DK : nullptr;
+#pragma unroll
+      for (int n = 0; n < N8; ++n) {
+        float2 x = make_float2(0.f, 0.f);
+        if (src) x = __ldcs(reinterpret_cast<const float2 *>(src + n * 8 + t2));
+        w[mt][n][2 * h] = x.x;
+        w[mt][n][2 * h + 1] = x.y;
+      }
+    }
+
+  // Iteration b: operands of block b+2 (converted, or on their way), Gram matrices of block b+1, then block b itself.
+#pragma unroll 1
+  for (int b = -2; b < nb; ++b) {
+    if (prepares && lane == 0) {
+      const int pwarp = ptid >> 5, parts = nt >= 128 ? 4 : 1;
+      if (pwarp < parts) {
+        fence_async_smem();
+        if (pwarp == 0) {
+          if constexpr (NPK == 1) {
+            if (b + 2 > 0 && b + 2 < nb) load_kq(b + 2);
+          } else {
+            if (b + 3 < nb) load_kq(b + 3);
+          }
+        }
+        // the gates of the next block, or, with one buffer, of this one: they are needed after its products with the state
+        const int bg = b + gate_bufs - 1;
+        if (bg >= 0 && bg < nb) load_gates(bg, pwarp, parts);
+      }
+    }
+    if (prepares) {
+      if constexpr (NPK == 3) {
+        if (b + 2 < nb) {
+          wait_kq(b + 2);
+          tile_convert<Cf>(smem + m.rawkq + (b & 1) * Cf::RAWKQ, smem + m.kq + ((b + 2) % Cf::NB) * 3 * Cf::PART, p.qkv_act, ptid, nt);
+        }
+      }
+      if (b + 1 >= 0 && b + 1 < nb) {
+        if constexpr (NPK == 1) wait_kq(b + 1);
+        const unsigned char *tile1 = smem + m.kq + ((b + 1) % Cf::NB) * NPK * Cf::PART;
+        float *gk1 = reinterpret_cast<float *>(smem + m.gk + ((b + 1) & 1) * Cf::GK);
+        unsigned char *gq1 = smem + m.gq + ((b + 1) & 1) * 3 * Cf::GQP;
+        for (int i = ptid >> 5; i < 4; i += nt >> 5) tile_gram<Cf>(tile1, i >> 1, i & 1, gk1, gq1, lane);
+      }
+    }
+    if (holds && b >= 0) {
+      const int nvalid = min(C, p.T - b * C);
+      const unsigned char *gates = smem + m.gates + (gate_bufs == 2 ? b & 1 : 0) * m.gates_stage;
+      const float *gk = reinterpret_cast<const float *>(smem + m.gk + (b & 1) * Cf::GK);
+      const uint32_t tile = smem_u32(smem + m.kq + (b % Cf::NB) * NPK * Cf::PART);
+      const uint32_t gq = smem_u32(smem + m.gq + (b & 1) * 3 * Cf::GQP);
+      unsigned char *xch = smem + m.xch + warp * Cf::XCH;
+      float *wb = reinterpret_cast<float *>(smem + m.wb + warp * Cf::WB);
+      if constexpr (NPK == 1) wait_kq(b);  // (completed before: it makes the copies visible to this thread)
+
+      // a 128-byte row holds 8 units; K step ks of a half of 64 key dims is the unit pair XORed with 2 ks
+      const uint32_t t1 = tile + tile_at(((lane >> 4) & 1) * 8 + (lane & 7), (lane >> 3) & 1);  // products with the state
+      const uint32_t t3 = tile + tile_at(((lane >> 3) & 1) * 8 + (lane & 7), lane >> 4);       // update, transposed
+      const size_t tok = tok0 + (size_t)b * C;
+      float r[MT][2][4];
+      // ---- p and r of the block: W (in parts) times the 32 vectors, two row tiles at a time ----
+#pragma unroll
+      for (int mp = 0; mp < MT; mp += 2) {
+        float acc[2][4][4];
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[x][n][e] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < KS; ++ks) {
+          uint32_t bq[NPK][2][4];
+#pragma unroll
+          for (int s = 0; s < NPK; ++s)
+#pragma unroll
+            for (int x = 0; x < 2; ++x)
+              tile_ldsm(bq[s][x], (t1 ^ ((ks & 3) * 32)) + s * Cf::PART + x * 2048 + (ks >> 2) * 4096);
+#pragma unroll
+          for (int x = 0; x < 2; ++x) {
+            const float(&w0)[4] = w[mp + x][2 * ks], (&w1)[4] = w[mp + x][2 * ks + 1];
+            uint32_t q[4][Cf::NPW];
+            tile_split(w0[0], w0[1], q[0]);
+            tile_split(w0[2], w0[3], q[1]);
+            tile_split(w1[0], w1[1], q[2]);
+            tile_split(w1[2], w1[3], q[3]);
+#pragma unroll
+            for (int pa = Cf::NPW - 1; pa >= 0; --pa)
+#pragma unroll
+              for (int s = 0; s < NPK; ++s)
+                if (pa + s < Cf::NPW) {
+                  const uint32_t a[4] = {q[0][pa], q[1][pa], q[2][pa], q[3][pa]};
+#pragma unroll
+                  for (int n = 0; n < 4; ++n) tile_mma(acc[x][n], a, bq[s][n >> 1][(n & 1) * 2], bq[s][n >> 1][(n & 1) * 2 + 1]);
+                }
+          }
+        }
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          unsigned char *xr = xch + ((mp + x) * 16 + g) * Cf::XROW + t2 * 4;
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) *reinterpret_cast<float2 *>(xr + h * 8 * Cf::XROW + n * 32) = make_float2(acc[x][n][2 * h], acc[x][n][2 * h + 1]);
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) r[mp + x][n][e] = acc[x][n + 2][e];
+        }
+      }
+      __syncwarp();
+
+      // ---- token by token, in two trips of eight.  Rolled: the loop over the blocks has to stay inside the instruction cache (with
+      //      64 rows per warp and 16 tokens straight it is fetched at three quarters of the GPC cache's rate) ----
+      {
+        float2 P2[RL][C / 2];
+        unsigned char *row[RL];
+#pragma unroll
+        for (int i = 0; i < RL; ++i) {
+          row[i] = xch + ((ln.comp0 + i % Cf::CL) * CPW + ln.col + (i / Cf::CL) * Cf::LCOLS) * Cf::XROW;
+#pragma unroll
+          for (int q = 0; q < C / 4; ++q) {
+            const float4 y = reinterpret_cast<const float4 *>(row[i])[q];
+            P2[i][2 * q] = make_float2(y.x, y.y);
+            P2[i][2 * q + 1] = make_float2(y.z, y.w);
+          }
+        }
+        wait(3 + (b & 1), (b >> 1) & 1);
+        const uint32_t gates_s = smem_u32(gates), gk_s = smem_u32(gk);
+        const int colr = col0 + wcol + ln.col;
+        TileGates<Cf> gt;
+        gt.prime(p, m, ln, gates_s, cols, wcol, 0, nvalid);
+#pragma unroll 1
+        for (int tg = 0; tg < C; tg += 8) {
+          [[maybe_unused]] TileLane<Cf> before;
+          if constexpr (Cf::EXT) before = ln;
+          const bool bad = tile_trip<Cf, false>(p, m, ln, gt, P2, gk_s, cols + Cf::PAD, tg, nvalid, colr, tok);
+          if (__any_sync(0xffffffffu, bad)) {
+            if constexpr (Cf::EXT) {
+              ln = before;
+              const int slots = tg == 0 ? C : 8;
+#pragma unroll
+              for (int i = 0; i < RL; ++i)
+#pragma unroll
+                for (int u = 0; u < C / 2; ++u) P2[i][u] = 2 * u < slots ? reinterpret_cast<const float2 *>(row[i] + tg * 4)[u] : make_float2(0.f, 0.f);
+              TileGates<Cf> again;
+              again.prime(p, m, ln, gates_s, cols, wcol, tg, nvalid);
+              tile_trip<Cf, true>(p, m, ln, again, P2, gk_s, cols + Cf::PAD, tg, nvalid, colr, tok);
+            } else {
+              tile_trip_again<Cf>(&p, &m, xch, gates_s, gk_s, cols, wcol, tg, nvalid, colr, tok);
+              const int slots = tg == 0 ? C : 8;
+#pragma unroll
+              for (int i = 0; i < RL; ++i)
+#pragma unroll
+                for (int u = 0; u < C / 2; ++u) P2[i][u] = 2 * u < slots ? reinterpret_cast<const float2 *>(row[i] + tg * 4)[u] : make_float2(0.f, 0.f);
+            }
+          }
+          // the trip's coefficients in parts, the later predictions (for a trip that has to be run again), the window moves on
+#pragma unroll
+          for (int i = 0; i < RL; ++i) {
+            uint32_t c[4][3];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) tile_split(P2[i][n].x, P2[i][n].y, c[n]);
+            unsigned char *dst = row[i] + tg * 4;
+            *reinterpret_cast<uint4 *>(dst) = make_uint4(c[0][0], c[1][0], c[2][0], c[3][0]);
+            *reinterpret_cast<uint4 *>(dst + 16) = make_uint4(c[0][1], c[1][1], c[2][1], c[3][1]);
+            *reinterpret_cast<uint4 *>(row[i] + 64 + tg * 2) = make_uint4(c[0][2], c[1][2], c[2][2], c[3][2]);
+            if (tg == 0) {
+              *reinterpret_cast<float4 *>(dst + 32) = make_float4(P2[i][4].x, P2[i][4].y, P2[i][5].x, P2[i][5].y);
+              *reinterpret_cast<float4 *>(dst + 48) = make_float4(P2[i][6].x, P2[i][6].y, P2[i][7].x, P2[i][7].y);
+            }
+#pragma unroll
+            for (int n = 0; n < 4; ++n) P2[i][n] = P2[i][n + 4];
+          }
+        }
+        if constexpr (Cf::EXT) tile_weights<Cf>(p, m, ln, gates, wb, cols, wcol, nvalid);
+      }
+      __syncwarp();
+
+      // ---- r += C (K Q^T masked), W += C K ----
+      {
+        uint32_t bg[Cf::RPARTS][4];
+#pragma unroll
+        for (int s = 0; s < Cf::RPARTS; ++s) tile_ldsm(bg[s], gq + s * Cf::GQP + (((lane >> 4) & 1) * 8 + (lane & 7)) * 48 + ((lane >> 3) & 1) * 16);
+        const uint32_t xa = smem_u32(xch) + ((lane & 7) + ((lane >> 3) & 1) * 8) * Cf::XROW;
+        const int half = lane >> 4;
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) {
+          uint32_t c[3][4];
+#pragma unroll
+          for (int s = 0; s < 3; ++s) tile_ldsm(c[s], xa + mt * 16 * Cf::XROW + (half ? tile_c_at(s, 1) : tile_c_at(s, 0)));
+#pragma unroll
+          for (int pa = Cf::RPARTS - 1; pa >= 0; --pa)
+#pragma unroll
+            for (int s = 0; s < Cf::RPARTS; ++s)
+              if (pa + s < Cf::RPARTS) {
+                tile_mma(r[mt][0], c[pa], bg[s][0], bg[s][1]);
+                tile_mma(r[mt][1], c[pa], bg[s][2], bg[s][3]);
+              }
+#pragma unroll
+          for (int n4 = 0; n4 < N8; n4 += 4) {  // four accumulator tiles at a time: independent chains
+            uint32_t bk[NPK][2][4];
+#pragma unroll
+            for (int s = 0; s < NPK; ++s)
+#pragma unroll
+              for (int x = 0; x < 2; ++x) tile_ldsm_t(bk[s][x], (t3 ^ (((n4 + 2 * x) & 7) * 16)) + s * Cf::PART + (n4 >> 3) * 4096);
+#pragma unroll
+            for (int pa = 2; pa >= 0; --pa)
+#pragma unroll
+              for (int s = 0; s < NPK; ++s)
+                if (pa + s < 3) {
+#pragma unroll
+                  for (int n = 0; n < 4; ++n) tile_mma(w[mt][n4 + n], c[pa], bk[s][n >> 1][(n & 1) * 2], bk[s][n >> 1][(n & 1) * 2 + 1]);
+                }
+          }
+        }
+      }
+
+      // ---- outputs (Eq. 3.5): a lane holds, for its tokens 8 n + t2 + {0, 1}, the rows g and g + 8 of every tile, which are NCS columns with
+      //      NCL components each; with fewer than 8 columns per warp the other components are in lanes GC apart in g ----
+      IO *ost = reinterpret_cast<IO *>(xch);
+      __syncwarp();  // the coefficients have been read by all lanes
+      {
+        const int grow = cols + Cf::PAD;
+        const int gcomp = g / Cf::GC, gcol = g % Cf::GC;
+        const IO *const io = nullptr;
+        const uint32_t gpq = smem_u32(gates) + m.g_pq + ((t2 * J + gcomp) * grow + wcol + gcol) * Cf::ES;
+        float xn[Cf::NCS][Cf::NCL];
+        auto fetch_pq = [&](int i) {  // token 8 (i / 2) + t2 + i % 2; component c * 8 / GC + gcomp, column 8 cs + gcol
+#pragma unroll
+          for (int cs = 0; cs < Cf::NCS; ++cs)
+#pragma unroll
+            for (int c = 0; c < Cf::NCL; ++c)
+              xn[cs][c] = tile_lds(gpq + (((8 * (i >> 1) + (i & 1)) * J + c * (8 / Cf::GC)) * grow + 8 * cs) * Cf::ES, io);
+        };
+        if (!temporal) fetch_pq(0);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int n = i >> 1, e = i & 1, t = 8 * n + t2 + e;
+          float x[Cf::NCS][Cf::NCL];
+#pragma unroll
+          for (int cs = 0; cs < Cf::NCS; ++cs)
+#pragma unroll
+            for (int c = 0; c < Cf::NCL; ++c) x[cs][c] = xn[cs][c] * kLog2e;
+          if (!temporal && i + 1 < 4) fetch_pq(i + 1);
+#pragma unroll
+          for (int cs = 0; cs < Cf::NCS; ++cs) {
+            float mx = x[cs][0], num = 0.f, den = 0.f;
+#pragma unroll
+            for (int c = 1; c < Cf::NCL; ++c) mx = fmaxf(mx, x[cs][c]);
+            if constexpr (Cf::GC < 8) {
+#pragma unroll
+              for (int off = Cf::GC; off < 8; off <<= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off * 4));
+            }
+#pragma unroll
+            for (int c = 0; c < Cf::NCL; ++c) {
+              const int rho = Cf::GC == 8 ? c * CPW + cs * 8 : c * 8;  // row of the tile stack, without g
+              const float rv = r[rho / 16][n][((rho / 8) & 1) * 2 + e];
+              if (temporal) {
+                num = fmaf(wb[(rho + g) * Cf::WROW + t], rv, num);
+              } else {
+                const float ex = ex2_approx(x[cs][c] - mx);
+                den += ex;
+                num = fmaf(ex, rv, num);
+              }
+            }
+            if constexpr (Cf::GC < 8) {
+#pragma unroll
+              for (int off = Cf::GC; off < 8; off <<= 1) {
+                num += __shfl_xor_sync(0xffffffffu, num, off * 4);
+                den += __shfl_xor_sync(0xffffffffu, den, off * 4);
+              }
+            }
+            if (Cf::GC == 8 || gcomp == 0) from_f32(ost[t * CPW + 8 * cs + gcol], temporal ? num : num * rcp_approx(den));
+          }
+        }
+      }
+      __syncwarp();
+      {
+        constexpr int VB = CPW * Cf::ES < 16 ? CPW * Cf::ES : 16, VE = VB / Cf::ES, VPT = CPW / VE;
+        for (int i = lane; i < nvalid * VPT; i += 32) {
+          const int t = i / VPT, c = (i - t * VPT) * VE, col = col0 + wcol + c;
+          if (col < p.Dv) {
+            IO *dst = (IO *)p.o + (tok + t) * p.Dv + col;
+            const IO *src = ost + t * CPW + c;
+            if constexpr (VB == 16) *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
+            else if constexpr (VB == 8) *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(src);
+            else *reinterpret_cast<uint32_t *>(dst) = *reinterpret_cast<const uint32_t *>(src);
+          }
+        }
+      }
+    }
+    __syncthreads();
+  }
+
+  // ---- accumulator tiles -> state, carried distributions, statistics ----
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int rho = mt * 16 + h * 8 + g, comp = rho / CPW, col = col0 + wcol + rho % CPW;
+      if (p.W_out && holds && col < p.Dv) {
+        float *dst = p.W_out + (((size_t)bh * J + comp) * p.Dv + col) * DK;
+#pragma unroll
+        for (int n = 0; n < N8; ++n) __stcs(reinterpret_cast<float2 *>(dst + n * 8 + t2), make_float2(w[mt][n][2 * h], w[mt][n][2 * h + 1]));
+      }
+    }
+  if constexpr (Cf::EXT) {
+    constexpr float kLn2 = 0.6931471805599453f;
+#pragma unroll
+    for (int o = 0; o < Cf::OCL; ++o) {
+      const int col = col0 + wcol + ln.col + o * Cf::LCOLS;
+      float hr = 0.f, hq = 0.f;
+#pragma unroll
+      for (int c = 0; c < Cf::CL; ++c) { hr += ln.s_rh[o * Cf::CL + c]; hq += ln.s_qh[o * Cf::CL + c]; }
+      hr = tile_over_j<Cf>(hr, TileAdd());
+      hq = tile_over_j<Cf>(hq, TileAdd());
+      if (!holds || col >= p.Dv) continue;  // (the shuffles are above)
+#pragma unroll
+      for (int c = 0; c < Cf::CL; ++c) {
+        const int r = o * Cf::CL + c;
+        const size_t at = ((size_t)bh * J + ln.comp0 + c) * p.Dv + col;
+        if (temporal && p.r_out) p.r_out[at] = ln.rp[r];
+        if (temporal && p.rho_out) p.rho_out[at] = ln.rho[r];
+        // each element belongs to one lane of one block: plain read-modify-write
+        if (p.r_sum) p.r_sum[at] += ln.s_r[r];
+        if (p.rho_sum) p.rho_sum[at] += ln.s_q[r];
+      }
+      const size_t ate = (size_t)bh * p.Dv + col;
+      if (ln.comp0 == 0 && p.r_ent) p.r_ent[ate] -= hr * kLn2;
+      if (ln.comp0 == 0 && p.rho_ent) p.rho_ent[ate] -= hq * kLn2;
+    }
+  }
+}
+
+// ---- host-side launch of one instantiation -----------------------------------------------
+template <class Cf>
+bool tile_make_maps(const ScanParams &p, int cols, TileMaps *m) {
+  const cuuint64_t BH = (cuuint64_t)p.B * p.H, T = (cuuint64_t)p.T, Dv = (cuuint64_t)p.Dv, J = Cf::J, DK = Cf::DK, es = Cf::ES;
+  const CUtensorMapDataType io = es == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+  auto rows = [&](CUtensorMap *map, const void *base, cuuint64_t width, int box_width, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_NONE) {  // [BH][T][width]
+    const cuuint64_t dims[3] = {width, T, BH}, strides[2] = {width * es, T * width * es};
+    const cuuint32_t box[3] = {(cuuint32_t)box_width, (cuuint32_t)Cf::C, 1};
+    return tma_encode(map, base, 3, dims, strides, box, swizzle, io);
+  };
+  auto gates = [&](CUtensorMap *map, const void *base) {  // [BH][T][J][Dv]
+    const cuuint64_t dims[4] = {Dv, J, T, BH}, strides[3] = {Dv * es, J * Dv * es, T * J * Dv * es};
+    const cuuint32_t box[4] = {(cuuint32_t)(cols + Cf::PAD), (cuuint32_t)J, (cuuint32_t)Cf::C, 1};
+    return tma_encode(map, base, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE, io);
+  };
+  const CUtensorMapSwizzle kq = Cf::NPK == 1 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE;
+  const int kq_box = Cf::NPK == 1 ? 64 : Cf::DK;
+  bool ok = rows(&m->k, p.k, DK, kq_box, kq) && rows(&m->q, p.q, DK, kq_box, kq) && rows(&m->v, p.v, Dv, cols);
+  ok = ok && gates(&m->be, p.beta_logit) && gates(&m->pk, p.pik_logit) && gates(&m->pq, p.piq_logit);
+  if (p.temporal) ok = ok && rows(&m->gk, p.gk_logit, Dv, cols) && rows(&m->gq, p.gq_logit, Dv, cols);
+  return ok;
+}
+
+// Warps (CPW columns each) per thread block: as many as share the operand preparation usefully, fewer where even then every
+// block has an SM to itself.  A slice is a multiple of 8 columns and a copy box has at most 256.
+template <class Cf>
+int tile_warps(const ScanParams &p, int sms) {
+  const long long bh = (long long)p.B * p.H;
+  int nw = 1;
+  while (nw < 4 && nw * Cf::CPW < p.Dv && 2 * nw * Cf::CPW + Cf::PAD <= 256) nw *= 2;
+  while (nw > 1 && (nw / 2 * Cf::CPW) % 8 == 0 && bh * ((p.Dv + nw / 2 * Cf::CPW - 1) / (nw / 2 * Cf::CPW)) <= sms) nw /= 2;
+  while ((nw * Cf::CPW) % 8 != 0) nw *= 2;
+  return nw;
+}
+
+template <class Cf>
+int launch_tile(const LaunchArgs &a, int *err, int sms) {
+  const int nw = tile_warps<Cf>(a.p, sms), cols = nw * Cf::CPW;
+  const long long grid = (long long)a.p.B * a.p.H * ((a.p.Dv + cols - 1) / cols);
+  // One block per SM or less: four more warps take the preparation off the state warps, and the gates are fetched a block ahead.
+  // More blocks: they hide each other's waits, and shared memory decides how many are resident.
+  const int prep = grid <= sms ? 4 : 0, gate_bufs = grid <= sms ? 2 : 1;
+  const TileSmem m = tile_smem<Cf>(nw, a.p.temporal != 0, gate_bufs);
+  if (m.total > 227 * 1024) return -1000;
+  if (grid <= 0 || grid > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
+  TileMaps maps;
+  if (!tile_make_maps<Cf>(a.p, cols, &maps)) return (int)cudaErrorInvalidValue;
+  auto kern = swila_tile_kernel<Cf>;
+  static std::atomic<uint64_t> granted;
+  cudaError_t e = allow_smem((const void *)kern, 227 * 1024, granted);  // (the size differs from launch to launch)
+  if (e != cudaSuccess) return (int)e;
+  kern<<<(unsigned)grid, (nw + prep) * 32, m.total, a.stream>>>(a.p, maps, nw, gate_bufs, err);
+  return (int)cudaGetLastError();
+}
+
+}  // namespace swila

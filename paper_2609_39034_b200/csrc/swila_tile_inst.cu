@@ -1,0 +1,49 @@
+// Instantiations of the register-tile kernel: one translation unit per (key dimension, io dtype), compiled with
+// -DSWILA_DK=<64|128> -DSWILA_BF16=<0|1>.
+#include "swila_tile.cuh"
+
+#ifndef SWILA_DK
+#error "compile with -DSWILA_DK, -DSWILA_BF16"
+#endif
+
+namespace swila {
+
+namespace {
+template <int J, bool EXT, int NPK>
+int pick(const LaunchArgs &a, int *err, int sms) {
+#if SWILA_BF16
+  using IO = __nv_bfloat16;
+#else
+  using IO = float;
+#endif
+  // two row tiles per warp: 64 state registers per lane at Dk = 64, 128 at Dk = 128
+  return launch_tile<TileCfg<IO, J, SWILA_DK, 2, EXT, NPK>>(a, err, sms);
+}
+template <bool EXT>
+int pick_j(const LaunchArgs &a, int *err, int sms) {
+#define SWILA_CASE(JJ)                                                             \
+  case JJ:                                                                         \
+    if constexpr (SWILA_BF16 && JJ != 4 && JJ != 8) { /* (those are the chunked kernel's) */ \
+      if (!a.p.qkv_act) return pick<JJ, EXT, 1>(a, err, sms);                      \
+    }                                                                              \
+    return pick<JJ, EXT, 3>(a, err, sms);
+  switch (a.J) {
+    SWILA_CASE(1)
+    SWILA_CASE(2)
+    SWILA_CASE(4)
+    SWILA_CASE(8)
+    SWILA_CASE(16)
+    default: return -1000;
+  }
+#undef SWILA_CASE
+}
+}  // namespace
+
+// Returns a cudaError_t value (>= 0), or -1000 when the combination is not compiled.
+template <>
+int tile_dispatch<SWILA_DK, (SWILA_BF16 != 0)>(const LaunchArgs &a, int *err, int sms) {
+  const bool ext = a.p.temporal || a.p.r_debug || a.p.r_sum || a.p.r_ent || a.p.rho_sum || a.p.rho_ent;
+  return ext ? pick_j<true>(a, err, sms) : pick_j<false>(a, err, sms);
+}
+
+}  // namespace swila

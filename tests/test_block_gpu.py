@@ -1,0 +1,98 @@
+"""GPU parity of the blocked scan (what AUTO takes from 64 tokens on where the chunked kernel does not apply) against the
+fp64 CPU oracle, where it can go wrong: partial token blocks, partial column slices, every lane split, each decay mode and
+what goes with it."""
+import pytest
+import torch
+
+from paper_2609_39034_b200 import workloads as wl
+from tests._gpu_util import TOL_BF16_O, TOL_FP32, TOL_STATE, assert_close, gpu_forward, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def binding():
+    assert torch.cuda.is_available(), "these tests need a CUDA device"
+    from paper_2609_39034_b200 import binding as b
+
+    return b
+
+
+def _w(D, J, io, T, Dv=None, B=1, H=2):
+    return wl.Workload(f"d{D}_j{J}_{io}_t{T}_v{Dv or D}", 1, B=B, H=H, T=T, Dk=D, Dv=Dv or D, J=J, io_dtype=io)
+
+
+SHAPES = [_w(16, 1, "fp32", 64), _w(16, 2, "fp32", 71, Dv=24), _w(16, 4, "bf16", 65, Dv=8), _w(16, 8, "fp32", 66), _w(16, 16, "bf16", 79),
+          _w(64, 1, "fp32", 64, Dv=264), _w(64, 2, "bf16", 70, Dv=72), _w(64, 4, "fp32", 129, Dv=40), _w(64, 8, "fp32", 100, B=2, H=3),
+          _w(64, 16, "fp32", 67), _w(128, 1, "bf16", 73), _w(128, 2, "fp32", 64, Dv=136), _w(128, 4, "fp32", 90), _w(128, 8, "fp32", 68, Dv=24),
+          _w(128, 16, "bf16", 69, H=1)]
+VARIANTS = [dict(), dict(temporal=True), dict(gated=True), dict(gated=True, post_decay=True), dict(gated=True, temporal=True),
+            dict(gated=True, granularity=wl.GRAN_PER_OUT), dict(gated=True, granularity=wl.GRAN_PER_OUT, post_decay=True),
+            dict(gated=True, granularity=wl.GRAN_SCALAR, temporal=True)]
+
+
+@pytest.mark.parametrize("w0", SHAPES, ids=lambda w: w.name)
+@pytest.mark.parametrize("var", VARIANTS, ids=lambda v: "+".join(f"{k}={v[k]}" for k in v) or "plain")
+def test_blocked_scan_matches_oracle(binding, oracle, w0, var):
+    w = w0.variant(**var)
+    inp = wl.make_inputs(w, stress=True)
+    ref = oracle.forward_inputs(inp, flags=w.flags, gran=w.gate_granularity, want_r=True)
+    dev = to_dev(inp)
+    got = gpu_forward(binding, w, dev, want_r=True)  # the instantiation with auxiliary outputs
+    plain = gpu_forward(binding, w, dev)
+    binding.device_status()
+    assert_close(w, got, ref, w.name)
+    if binding.auto_algo(w, aux_outputs=False) == binding.ALGO_SCAN:
+        assert torch.equal(got["o"], plain["o"]) and torch.equal(got["W"], plain["W"])
+    scan = gpu_forward(binding, w, dev, algo=binding.ALGO_SCAN)
+    if not (w.Dk == 128 and w.J == 16 and w.gated):
+        assert not torch.equal(scan["W"], plain["W"])  # it was not the sequential scan that ran
+
+
+@pytest.mark.parametrize("w0", [SHAPES[1], SHAPES[7], SHAPES[12]], ids=lambda w: w.name)
+@pytest.mark.parametrize("post", [False, True], ids=["pre", "post"])
+def test_blocked_scan_with_vanishing_decays(binding, oracle, w0, post):
+    """Decays per key dimension down to zero: the Gram matrices may not divide by their product then."""
+    w = w0.variant(gated=True, post_decay=post)
+    inp = wl.make_inputs(w, stress=True)
+    a = inp["alpha"].clone()
+    a[:, :, 17:30, 0, 3] = 1e-4
+    a[:, :, 40, :, 7] = 0.0
+    a[:, :, w.T - 1, w.J - 1, :] = 0.0
+    inp["alpha"] = a
+    ref = oracle.forward_inputs(inp, flags=w.flags, gran=w.gate_granularity)
+    assert_close(w, gpu_forward(binding, w, to_dev(inp)), ref, w.name)
+
+
+@pytest.mark.parametrize("var", [dict(), dict(temporal=True), dict(gated=True)], ids=["plain", "temporal", "gated"])
+def test_blocked_scan_far_from_the_noise_scale(binding, oracle, var):
+    """Every Gaussian factor underflows in FP32: the block is evaluated again with the maximum subtracted.  |delta| of 40 costs
+    the exponent eleven bits, so the bound is what the sequential scan, likewise in FP32, is off by on the same input."""
+    w = _w(64, 4, "fp32", 100).variant(**var)
+    inp = wl.make_inputs(w, stress=True)
+    inp["v"][:, :, 10:13] *= 40.0
+    inp["v"][:, :, 95] = -48.0
+    inp["piq_logit"][:, :, 30] *= 60.0
+    ref = oracle.forward_inputs(inp, flags=w.flags, gran=w.gate_granularity)
+    got, scan = (gpu_forward(binding, w, to_dev(inp), algo=a) for a in (binding.ALGO_AUTO, binding.ALGO_SCAN))
+    for n in ("W", "o"):
+        off, scan_off = (wl.rel_err(x[n], torch.from_numpy(ref[n])) for x in (got, scan))
+        print(n, off, scan_off)
+        assert off < 2e-3 + 4 * scan_off, (n, off, scan_off)
+
+
+@pytest.mark.parametrize("var", [dict(), dict(gated=True), dict(temporal=True)], ids=["plain", "gated", "temporal"])
+@pytest.mark.parametrize("D,J,io", [(64, 4, "bf16"), (128, 2, "fp32"), (16, 4, "fp32")])
+def test_blocked_scan_activates_raw_projections(binding, oracle, var, D, J, io):
+    from oracle import swila_fusions as fus
+
+    w = _w(D, J, io, 77).variant(**var)
+    inp = wl.make_inputs(w, stress=True)
+    g = torch.Generator().manual_seed(3)
+    for n in ("q", "k", "v"):
+        inp[n] = torch.randn(inp[n].shape, generator=g).to(w.torch_io_dtype)
+    qa, ka, va = fus.qkv_activation(inp["q"], inp["k"], inp["v"])
+    ref = oracle.forward_inputs(dict(inp, q=qa, k=ka, v=va), flags=w.flags, gran=w.gate_granularity)
+    got = gpu_forward(binding, w.with_(flags=w.flags | wl.FLAG_QKV_ACT), to_dev(inp))
+    assert wl.rel_err(got["o"], torch.from_numpy(ref["o"])) < (TOL_BF16_O if io == "bf16" else TOL_FP32)
+    assert wl.rel_err(got["W"], torch.from_numpy(ref["W"])) < TOL_STATE
