@@ -55,16 +55,15 @@ struct BlockCfg {
   static constexpr int NKQ = GATE == 1 ? 2 : 3;                                 // ring of converted blocks
   static constexpr int RW = CG * J * NC;                                        // rows per warp
   static constexpr int NCOPY = OC == 1 ? 2 : 1;                                 // orders the coefficients are stored in
-  // a warp's exchange buffer, floats: first every lane's p_t, r_t, then the update coefficients of the warp's rows
-  static constexpr int CB1 = (C + (GATE == 2 ? 1 : 0)) * NCOPY * RW * 2, CB2 = C * 2 * OC * 32;
-  static constexpr int CB = CB1 > CB2 ? CB1 : CB2;
+  // a warp's exchange buffers, floats: the update coefficients of its rows, and every lane's p_t, r_t
+  static constexpr int CB = (C + (GATE == 2 ? 1 : 0)) * NCOPY * RW * 2, XCH = C * 2 * OC * 32;
 };
 
 __host__ __device__ constexpr int block_up128(int n) { return (n + 127) & ~127; }
 
 // Shared-memory map of a launch (bytes); the number of columns per thread block is a launch parameter.
 struct BlockSmem {
-  int rawkq, rawkq_stage, alpha, alpha_stage, gates, gates_stage, g_be, g_pk, g_pq, g_gk, g_gq, g_ar, kq, kt, kb, kh, ac, gram, cbuf, ost, bars, total;
+  int rawkq, rawkq_stage, alpha, alpha_stage, gates, gates_stage, g_be, g_pk, g_pq, g_gk, g_gq, g_ar, kq, kt, kb, kh, ac, gram, cbuf, xch, ost, bars, total;
 };
 template <class Cf>
 __host__ __device__ inline BlockSmem block_smem(int nwarps, bool temporal, bool row_alpha) {
@@ -86,6 +85,7 @@ __host__ __device__ inline BlockSmem block_smem(int nwarps, bool temporal, bool 
   m.ac = off; off += 2 * Cf::J * Cf::AC * 4;
   m.gram = off; off += 2 * Cf::GJ * Cf::GR * 4;
   m.cbuf = off; off += nwarps * Cf::CB * 4;
+  m.xch = off; off += nwarps * Cf::XCH * 4;
   m.ost = off; off += block_up128(nwarps * Cf::C * Cf::CPW * Cf::ES);
   m.bars = off; off += 64;
   m.total = off + 128;  // the kernel aligns its window to 128 bytes
@@ -138,6 +138,35 @@ __device__ __forceinline__ void block_ld(const IO *p, float (&x)[OC]) {
   } else {
 #pragma unroll
     for (int o = 0; o < OC; ++o) x[o] = to_f32(p[o]);
+  }
+}
+
+// The same from a shared-memory address, pinned where it is written (see lds_f32).
+template <typename IO, int OC>
+__device__ __forceinline__ void block_lds(uint32_t addr, float (&x)[OC]) {
+  if constexpr (OC % 2 == 0) {
+#pragma unroll
+    for (int o = 0; o < OC; o += 2) {
+      if constexpr (sizeof(IO) == 2) {
+        uint32_t u;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(u) : "r"(addr + o * 2));
+        x[o] = __uint_as_float(u << 16);
+        x[o + 1] = __uint_as_float(u & 0xffff0000u);
+      } else {
+        asm volatile("ld.shared.v2.f32 {%0,%1}, [%2];" : "=f"(x[o]), "=f"(x[o + 1]) : "r"(addr + o * 4));
+      }
+    }
+  } else {
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      if constexpr (sizeof(IO) == 2) {
+        unsigned short u;
+        asm volatile("ld.shared.u16 %0, [%1];" : "=h"(u) : "r"(addr + o * 2));
+        x[o] = __uint_as_float((uint32_t)u << 16);
+      } else {
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x[o]) : "r"(addr + o * 4));
+      }
+    }
   }
 }
 
@@ -290,16 +319,23 @@ struct BlockLane {
   float s_r[Cf::OC], s_rh[Cf::OC], s_q[Cf::OC], s_qh[Cf::OC];  // statistics (entropies in bits)
 };
 
-// Sum over the J lanes of a column (distance G).
-template <class Cf>
-__device__ __forceinline__ float block_sum_j(float x) {
+// Over the J lanes of a column (distance G); `shadow` is run once, behind the first shuffles.
+struct BlockNothing { __device__ __forceinline__ void operator()() const {} };
+template <class Cf, class Shadow = BlockNothing>
+__device__ __forceinline__ float block_sum_j(float x, Shadow shadow = Shadow()) {
   if constexpr (Cf::J == 4) {  // three independent shuffles: shorter than two dependent rounds
     const float a = __shfl_xor_sync(0xffffffffu, x, Cf::G), b = __shfl_xor_sync(0xffffffffu, x, 2 * Cf::G);
     const float c = __shfl_xor_sync(0xffffffffu, x, 3 * Cf::G);
+    shadow();
     return (x + a) + (b + c);
   } else {
 #pragma unroll
-    for (int off = 1; off < Cf::J; off <<= 1) x += __shfl_xor_sync(0xffffffffu, x, off * Cf::G);
+    for (int off = 1; off < Cf::J; off <<= 1) {
+      const float y = __shfl_xor_sync(0xffffffffu, x, off * Cf::G);
+      if (off == 1) shadow();
+      x += y;
+    }
+    if (Cf::J == 1) shadow();
     return x;
   }
 }
@@ -310,103 +346,147 @@ __device__ __forceinline__ float block_max_j(float x) {
   return x;
 }
 
+// Where a lane's update coefficients go: to the lanes of its row, each as a pair of equal values, ready for the packed FMAs, and,
+// when neighbouring registers of a lane may hold neighbouring columns in either order (OC = 1), in both orders.
+template <class Cf>
+struct BlockPut {
+  static constexpr int TS = Cf::NCOPY * Cf::RW * 2;  // floats per token
+  float *w, *other;
+  __device__ __forceinline__ BlockPut(float *cb, const BlockLane<Cf> &ln) {
+    const int rowb = (ln.cg * Cf::J + ln.j) * Cf::NC;
+    w = cb + (rowb + ln.mask) * 2;
+    other = cb + (Cf::RW + rowb + (ln.mask ^ 1)) * 2;
+  }
+  __device__ __forceinline__ void operator()(int t, int o, float x) const {
+    *reinterpret_cast<float2 *>(w + t * TS + o * 2) = make_float2(x, x);
+    if constexpr (Cf::NCOPY == 2) *reinterpret_cast<float2 *>(other + t * TS) = make_float2(x, x);
+  }
+};
+
 // Entered with the lane's p_t and r_t of the block in `xch` ([t][lane][p of OC columns, r of OC columns]); hands every update
-// coefficient to put(t, o, c) and writes the outputs to `ost` ([C][CPW], io dtype).  EXACT subtracts the maximum before every exponential; without it the pass
-// returns true when a normaliser left the safe range, and the caller runs the block again.
-template <class Cf, bool EXACT, class Put>
-__device__ __forceinline__ bool block_tokens(const ScanParams &p, const BlockSmem &m, BlockLane<Cf> &ln, const float *xch, Put put,
+// coefficient to put(t, o, c) and writes the outputs to `ost` ([C][CPW], io dtype).  EXACT subtracts the maximum before every
+// exponential; without it the pass returns true when a normaliser left the safe range, and the caller runs the block again.
+//
+// What bounds it: the serial chain of a token (two exponential-unit instructions, one round of shuffles) and its instructions.  Loads are
+// pinned under the latency of the shuffles, one token ahead: free to move them, the compiler fetches the gates of all tokens first and spills
+// the state.
+template <class Cf, bool EXACT>
+__device__ __forceinline__ bool block_tokens(const ScanParams &p, const BlockSmem &m, BlockLane<Cf> &ln, const float *xch, const BlockPut<Cf> &put,
                                              const unsigned char *gates, const float *gram, typename Cf::IO *ost, int cols, int nvalid, int col,
                                              size_t tok) {
   using IO = typename Cf::IO;
-  constexpr int J = Cf::J, C = Cf::C, OC = Cf::OC, G = Cf::G;
+  constexpr int J = Cf::J, C = Cf::C, OC = Cf::OC, G = Cf::G, ES = Cf::ES;
   const int grow = cols + Cf::PAD;
   const bool temporal = Cf::EXT && p.temporal != 0;
-  const IO *gv = reinterpret_cast<const IO *>(gates) + ln.lc;
-  const IO *gbe = reinterpret_cast<const IO *>(gates + m.g_be) + ln.j * grow + ln.lc;
-  const IO *gpk = reinterpret_cast<const IO *>(gates + m.g_pk) + ln.j * grow + ln.lc;
-  const IO *gpq = reinterpret_cast<const IO *>(gates + m.g_pq) + ln.j * grow + ln.lc;
-  [[maybe_unused]] const IO *ggk = reinterpret_cast<const IO *>(gates + m.g_gk) + ln.lc;
-  [[maybe_unused]] const IO *ggq = reinterpret_cast<const IO *>(gates + m.g_gq) + ln.lc;
-  [[maybe_unused]] const float *gar = reinterpret_cast<const float *>(gates + m.g_ar) + ln.j * (cols + 4) + ln.lc;
+  const uint32_t gates_s = umma::smem_u32(gates), gram_s = umma::smem_u32(gram), xch_s = umma::smem_u32(xch);
+  const int sv = cols * ES, sg = J * grow * ES;  // bytes from token to token
+  uint32_t av = gates_s + ln.lc * ES, ag = gates_s + (ln.j * grow + ln.lc) * ES;
+  [[maybe_unused]] uint32_t at_gk = gates_s + m.g_gk + ln.lc * ES, at_ar = gates_s + m.g_ar + (ln.j * (cols + 4) + ln.lc) * 4;
+  const uint32_t apq = ag + m.g_pq, agq = gates_s + m.g_gq + ln.lc * ES;
   auto P = [&](float2(&x)[OC][C / 2], int o, int t) -> float & { return (t & 1) ? x[o][t >> 1].y : x[o][t >> 1].x; };
   float2 P2[OC][C / 2], R2[OC][C / 2];
 #pragma unroll
   for (int t = 0; t < C; ++t) {
     float x[2 * OC];
-    if constexpr (OC == 1) {
-      const float2 y = *reinterpret_cast<const float2 *>(xch + t * 64);
-      x[0] = y.x; x[1] = y.y;
-    } else {
-#pragma unroll
-      for (int i = 0; i < OC / 2; ++i) {
-        const float4 y = *reinterpret_cast<const float4 *>(xch + t * 64 * OC + 4 * i);
-        x[4 * i] = y.x; x[4 * i + 1] = y.y; x[4 * i + 2] = y.z; x[4 * i + 3] = y.w;
-      }
-    }
+    block_lds<float, 2 * OC>(xch_s + t * 256 * OC, x);
 #pragma unroll
     for (int o = 0; o < OC; ++o) { P(P2, o, t) = x[o]; P(R2, o, t) = x[OC + o]; }
   }
-  __syncwarp();  // the buffer is about to take the coefficients
   bool bad = false;
   float rp[OC], s_r[OC], s_rh[OC];
 #pragma unroll
   for (int o = 0; o < OC; ++o) { rp[o] = ln.rp[o]; s_r[o] = s_rh[o] = 0.f; }
 
-  float v[C][OC];
-#pragma unroll
-  for (int t = 0; t < C; ++t) block_ld<IO, OC>(gv + t * cols, v[t]);
-  if (p.qkv_act) {
-#pragma unroll
-    for (int t = 0; t < C; ++t)
-#pragma unroll
-      for (int o = 0; o < OC; ++o) v[t][o] = silu_approx(v[t][o]);
-  }
-
-#pragma unroll
-  for (int t = 0; t < C; ++t) {
-    float be[OC], lk[OC];
-    block_ld<IO, OC>(gbe + t * J * grow, be);
-    block_ld<IO, OC>(gpk + t * J * grow, lk);
-    [[maybe_unused]] float ar[OC];
+  // gates one token ahead: raw, then activated
+  float v_raw[OC], b_raw[OC], k_raw[OC], v[OC], be[OC], lk[OC];
+  [[maybe_unused]] float g_raw[OC], gt[OC], a_raw[OC], ar[OC];
+  auto fetch = [&](int t) {
+    block_lds<IO, OC>(av, v_raw);
+    block_lds<IO, OC>(ag + m.g_be, b_raw);
+    block_lds<IO, OC>(ag + m.g_pk, k_raw);
+    if (temporal) block_lds<IO, OC>(at_gk, g_raw);
     if constexpr (Cf::GATE == 2) {
-      // one decay per row: everything that is still to be used is decayed as the state would be
       if (p.gran == SWILA_GATE_PER_OUT) {
-        block_ld<float, OC>(gar + t * J * (cols + 4), ar);
+        block_lds<float, OC>(at_ar, a_raw);
       } else {
         const float a = t < nvalid ? __ldg(p.alpha + (tok + t) * J + ln.j) : 1.f;
 #pragma unroll
-        for (int o = 0; o < OC; ++o) ar[o] = a;
+        for (int o = 0; o < OC; ++o) a_raw[o] = a;
       }
-#pragma unroll
-      for (int o = 0; o < OC; ++o) {
-        if (t >= nvalid) ar[o] = 1.f;
-        if (!p.post) P(P2, o, t) *= ar[o];
-      }
+      at_ar += J * (cols + 4) * 4;
     }
-    float e[OC], c[OC];
+    av += sv; ag += sg; at_gk += sv;
+  };
+  auto activate = [&](int t) {
 #pragma unroll
     for (int o = 0; o < OC; ++o) {
-      be[o] = sigmoid_approx(be[o]);
+      v[o] = p.qkv_act ? silu_approx(v_raw[o]) : v_raw[o];
+      be[o] = sigmoid_approx(b_raw[o]);
       if (t >= nvalid) be[o] = 0.f;  // past the end of the sequence: no update
-      const float delta = v[t][o] - P(P2, o, t);
-      float a;
-      if (temporal) {
-        // prior (1 - g) r_{t-1} + g pi^k, pi^k normalised (App. B.3)
-        const float x = lk[o] * kLog2e, ex = ex2_approx(x - block_max_j<Cf>(x));
-        const float pk = ex * rcp_approx(block_sum_j<Cf>(ex));
-        float gk[OC];
-        block_ld<IO, OC>(ggk + t * cols, gk);
-        const float prior = fmaf(sigmoid_approx(gk[o]), pk - rp[o], rp[o]);
-        a = fmaf(-kHalfLog2e * delta, delta, lg2_approx(prior));
-      } else {
-        a = fmaf(-kHalfLog2e * delta, delta, lk[o] * kLog2e);
+      lk[o] = k_raw[o] * kLog2e;
+      if constexpr (Cf::GATE == 2) ar[o] = t < nvalid ? a_raw[o] : 1.f;
+      if (temporal) {  // the key-side prior enters a convex combination: normalised over the components (App. B.3)
+        gt[o] = sigmoid_approx(g_raw[o]);
+        const float ex = ex2_approx(lk[o] - block_max_j<Cf>(lk[o]));
+        lk[o] = ex * rcp_approx(block_sum_j<Cf>(ex));
       }
+    }
+  };
+  fetch(0);
+  activate(0);
+  fetch(1);
+  float gk[C], gq[C], cp[OC];  // one token's products with the later ones, its coefficients
+  auto push = [&](int t) {     // token t's pushes, its one into the next prediction aside
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      const float2 c2 = make_float2(cp[o], cp[o]);
+      if ((t & 1) && t + 2 < C) P(P2, o, t + 2) = fmaf(cp[o], gk[t + 2], P(P2, o, t + 2));
+#pragma unroll
+      for (int u = (t + 3) / 2; u < C / 2; ++u) P2[o][u] = fma2(c2, make_float2(gk[2 * u], gk[2 * u + 1]), P2[o][u]);
+      if (t & 1) P(R2, o, t) = fmaf(cp[o], gq[t], P(R2, o, t));
+#pragma unroll
+      for (int u = (t + 1) / 2; u < C / 2; ++u) R2[o][u] = fma2(c2, make_float2(gq[2 * u], gq[2 * u + 1]), R2[o][u]);
+    }
+  };
+#pragma unroll
+  for (int t = 0; t < C; ++t) {
+    float e[OC], c[OC];
+    [[maybe_unused]] float at[OC];
+    if constexpr (Cf::GATE == 2) {
+      // one decay per row: everything that is still to be used is decayed as the state would be.  (The previous token's pushes belong
+      // before the decay, so they are not deferred here.)
+#pragma unroll
+      for (int o = 0; o < OC; ++o) {
+        at[o] = ar[o];
+        if (!p.post) P(P2, o, t) *= at[o];
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < OC; ++o) {
+      const float prior = temporal ? lg2_approx(fmaf(gt[o], lk[o] - rp[o], rp[o])) : lk[o];  // log of (1 - g) r_{t-1} + g pi^k
+      const float delta = v[o] - P(P2, o, t), bd = be[o] * delta;
+      float a = fmaf(-kHalfLog2e * delta, delta, prior);
       if constexpr (EXACT) a -= block_max_j<Cf>(a);
       e[o] = ex2_approx(a);
-      const float sum = block_sum_j<Cf>(e[o]);
+      auto shadow = [&]() {
+        if (o + 1 < OC) return;
+        if (Cf::GATE != 2 && t > 0) push(t - 1);
+#pragma unroll
+        for (int i = 0; i < C / 4; ++i) {
+          if (4 * i + 3 > t) {
+            const float4 x = lds_f32x4<true>(gram + t * 2 * C + 4 * i);
+            gk[4 * i] = x.x; gk[4 * i + 1] = x.y; gk[4 * i + 2] = x.z; gk[4 * i + 3] = x.w;
+          }
+          if (4 * i + 3 >= t) {
+            const float4 x = lds_f32x4<true>(gram + t * 2 * C + C + 4 * i);
+            gq[4 * i] = x.x; gq[4 * i + 1] = x.y; gq[4 * i + 2] = x.z; gq[4 * i + 3] = x.w;
+          }
+        }
+      };
+      const float sum = block_sum_j<Cf>(e[o], shadow);
       if constexpr (!EXACT) bad = bad || !(sum > 1e-30f && sum < 1e30f);
       const float rs = rcp_approx(sum);
-      c[o] = ((be[o] * delta) * e[o]) * rs;
+      c[o] = (bd * e[o]) * rs;
       if constexpr (Cf::EXT) {
         const float r = e[o] * rs;
         if (t < nvalid) {
@@ -417,41 +497,26 @@ __device__ __forceinline__ bool block_tokens(const ScanParams &p, const BlockSme
         }
       }
     }
+    if (t + 1 < C) activate(t + 1);
+    if (t + 2 < C) fetch(t + 2);
     if constexpr (Cf::GATE == 2) {
 #pragma unroll
       for (int o = 0; o < OC; ++o) {
 #pragma unroll
-        for (int u = t + 1; u < C; ++u) P(P2, o, u) *= ar[o];
+        for (int u = t + 1; u < C; ++u) P(P2, o, u) *= at[o];
 #pragma unroll
-        for (int u = t; u < C; ++u) P(R2, o, u) *= ar[o];
-      }
-    }
-    // pushes into the later predictions and into the readouts from this token on
-    const float4 *gr = reinterpret_cast<const float4 *>(gram + t * 2 * C);
-    float gk[C], gq[C];
-#pragma unroll
-    for (int i = 0; i < C / 4; ++i) {
-      if (4 * i + 3 > t) {
-        const float4 x = gr[i];
-        gk[4 * i] = x.x; gk[4 * i + 1] = x.y; gk[4 * i + 2] = x.z; gk[4 * i + 3] = x.w;
-      }
-      if (4 * i + 3 >= t) {
-        const float4 x = gr[C / 4 + i];
-        gq[4 * i] = x.x; gq[4 * i + 1] = x.y; gq[4 * i + 2] = x.z; gq[4 * i + 3] = x.w;
+        for (int u = t; u < C; ++u) P(R2, o, u) *= at[o];
       }
     }
 #pragma unroll
     for (int o = 0; o < OC; ++o) {
+      if (t + 1 < C) P(P2, o, t + 1) = fmaf(c[o], gk[t + 1], P(P2, o, t + 1));  // the push that the next token waits for
       put(t, o, c[o]);
-      const float2 c2 = make_float2(c[o], c[o]);
-      if ((t & 1) == 0) P(P2, o, t + 1) = fmaf(c[o], gk[t + 1], P(P2, o, t + 1));
-#pragma unroll
-      for (int u = t / 2 + 1; u < C / 2; ++u) P2[o][u] = fma2(c2, make_float2(gk[2 * u], gk[2 * u + 1]), P2[o][u]);
-      if (t & 1) P(R2, o, t) = fmaf(c[o], gq[t], P(R2, o, t));
-#pragma unroll
-      for (int u = (t + 1) / 2; u < C / 2; ++u) R2[o][u] = fma2(c2, make_float2(gq[2 * u], gq[2 * u + 1]), R2[o][u]);
+      cp[o] = c[o];
     }
+    if (Cf::GATE == 2) push(t);
   }
+  if (Cf::GATE != 2) push(C - 1);
 
   // ---- readouts: o_t = sum_j pi^q_j (w_t.q_t)_j ----
   constexpr int N = C * OC;
@@ -462,7 +527,7 @@ __device__ __forceinline__ bool block_tokens(const ScanParams &p, const BlockSme
 #pragma unroll
   for (int t = 0; t < C; ++t) {
     float x[OC];
-    block_ld<IO, OC>(gpq + t * J * grow, x);
+    block_lds<IO, OC>(apq + t * sg, x);
 #pragma unroll
     for (int o = 0; o < OC; ++o) {
       x[o] *= kLog2e;
@@ -475,7 +540,7 @@ __device__ __forceinline__ bool block_tokens(const ScanParams &p, const BlockSme
         if (temporal) {
           w = e * rcp_approx(block_sum_j<Cf>(e));
           float gq[OC];
-          block_ld<IO, OC>(ggq + t * cols, gq);
+          block_lds<IO, OC>(agq + t * sv, gq);
           if (t < nvalid) rho[o] = fmaf(sigmoid_approx(gq[o]), w - rho[o], rho[o]);
           w = rho[o];
           num[t * OC + o] = w * P(R2, o, t);
@@ -535,6 +600,14 @@ __device__ __forceinline__ bool block_tokens(const ScanParams &p, const BlockSme
     }
   }
   return false;
+}
+
+// The exact pass out of line: rare, and its registers are not the fast path's.
+template <class Cf>
+__device__ __noinline__ void block_tokens_again(const ScanParams *p, const BlockSmem *m, const BlockLane<Cf> *lane, const float *xch, float *cb, const unsigned char *gates,
+                                                const float *gram, typename Cf::IO *ost, int cols, int nvalid, int col, size_t tok) {
+  BlockLane<Cf> ln = *lane;
+  block_tokens<Cf, true>(*p, *m, ln, xch, BlockPut<Cf>(cb, ln), gates, gram, ost, cols, nvalid, col, tok);
 }
 
 // ---- the kernel ---------------------------------------------------------------------------
@@ -684,18 +757,11 @@ __global__ void __launch_bounds__(256, Cf::L *Cf::NC <= 64 ? 2 : 1)
       const unsigned char *gates = smem + m.gates + (b & 1) * m.gates_stage;
       IO *ost = reinterpret_cast<IO *>(smem + m.ost) + warp * C * CPW;
       float *cb = reinterpret_cast<float *>(smem + m.cbuf) + warp * Cf::CB;
-      float *xch = cb + lane * 2 * OC;
-      // an update coefficient goes to the lanes of its row as a pair of equal values, ready for the packed FMAs, and, when
-      // neighbouring registers of a lane may hold neighbouring columns in either order (OC = 1), in both orders
-      constexpr int TS = Cf::NCOPY * Cf::RW * 2;  // floats per token
+      float *xch = reinterpret_cast<float *>(smem + m.xch) + warp * Cf::XCH + lane * 2 * OC;
+      const BlockPut<Cf> put(cb, ln);
+      constexpr int TS = BlockPut<Cf>::TS;
       const int rowb = (ln.cg * J + j) * NC;
-      float *cw = cb + (rowb + mask) * 2;
-      auto put = [&](int t, int o, float x) {
-        *reinterpret_cast<float2 *>(cw + t * TS + o * 2) = make_float2(x, x);
-        if constexpr (Cf::NCOPY == 2) *reinterpret_cast<float2 *>(cb + t * TS + (Cf::RW + rowb + (mask ^ 1)) * 2) = make_float2(x, x);
-      };
-#pragma unroll 1
-      for (int pass = 0; pass < 2; ++pass) {
+      {
         // state times k_t and q_t, reduced over the key slices.  The butterfly of token t-1 (val) runs between the FMAs of
         // token t, a round after each operand load.  The loop stays rolled: straight-line code for all tokens is fetched
         // slower than it is issued.
@@ -748,14 +814,17 @@ __global__ void __launch_bounds__(256, Cf::L *Cf::NC <= 64 ? 2 : 1)
 #pragma unroll
         for (int n = 0; n < L / 4; ++n) round(n);
         keep(C - 1);
-        __syncwarp();
-        if (pass == 0) {
-          wait(2, b);
-          if (!block_tokens<Cf, false>(p, m, ln, xch, put, gates, gram, ost, cols, nvalid, colw + mask, tok0 + (size_t)b * C)) break;
-        } else {
-          block_tokens<Cf, true>(p, m, ln, xch, put, gates, gram, ost, cols, nvalid, colw + mask, tok0 + (size_t)b * C);
+        wait(2, b);
+        const size_t tok = tok0 + (size_t)b * C;
+        if (block_tokens<Cf, false>(p, m, ln, xch, put, gates, gram, ost, cols, nvalid, colw + mask, tok)) {
+          if constexpr (Cf::EXT) {
+            block_tokens<Cf, true>(p, m, ln, xch, put, gates, gram, ost, cols, nvalid, colw + mask, tok);
+          } else {
+            const BlockLane<Cf> lane_copy = ln;  // (copies: the fast path's own may stay in registers)
+            const BlockSmem smem_copy = m;
+            block_tokens_again<Cf>(&p, &smem_copy, &lane_copy, xch, cb, gates, gram, ost, cols, nvalid, colw + mask, tok);
+          }
         }
-        __syncwarp();
       }
       if constexpr (GATE == 2) {  // c_t times the row's later decays; the product of all of them decays the state
         float sfx[OC];
@@ -772,7 +841,7 @@ __global__ void __launch_bounds__(256, Cf::L *Cf::NC <= 64 ? 2 : 1)
           }
 #pragma unroll
           for (int o = 0; o < OC; ++o) {
-            put(t, o, cw[t * TS + o * 2] * sfx[o]);
+            put(t, o, put.w[t * TS + o * 2] * sfx[o]);
             if (t < nvalid) sfx[o] *= a[o];
           }
         }
@@ -908,13 +977,13 @@ bool block_make_maps(const ScanParams &p, int cols, BlockMaps *m) {
 }
 
 // Warps (column slices of CPW) per thread block.  More warps share the operand preparation; fewer spread a small problem
-// over the SMs: halved while the grid would leave SMs without a block and the slice stays a multiple of 8 columns.
+// over the SMs: halved while every block still has an SM to itself and the slice stays a multiple of 8 columns.
 template <class Cf>
 int block_warps(const ScanParams &p, int sms) {
   const long long bh = (long long)p.B * p.H;
   int nw = 1;
   while (nw < 4 && nw * Cf::CPW < p.Dv && 2 * nw * Cf::CPW + Cf::PAD <= 256) nw *= 2;  // a copy box has at most 256 columns
-  while (nw > 1 && (nw / 2 * Cf::CPW) % 8 == 0 && bh * ((p.Dv + nw * Cf::CPW - 1) / (nw * Cf::CPW)) < sms) nw /= 2;
+  while (nw > 1 && (nw / 2 * Cf::CPW) % 8 == 0 && bh * ((p.Dv + nw / 2 * Cf::CPW - 1) / (nw / 2 * Cf::CPW)) <= sms) nw /= 2;
   while ((nw * Cf::CPW) % 8 != 0) nw *= 2;
   return nw;
 }
@@ -925,6 +994,10 @@ int launch_block(const LaunchArgs &a, int *err, int sms) {
   const BlockSmem m = block_smem<Cf>(nw, a.p.temporal != 0, Cf::GATE == 2 && a.p.gran == SWILA_GATE_PER_OUT);
   const long long grid = (long long)a.p.B * a.p.H * ((a.p.Dv + cols - 1) / cols);
   if (m.total > 227 * 1024) return -1000;
+  // Per-key decays need operands of every component: with Dk = 128, or eight components, that is one block per SM whatever the grid.  While
+  // the grid leaves it at that, the blocked form wins (1 x 16 heads, 2,048 tokens: Dk = 128 2,220 -> 1,446 us, J = 8 2,364 -> 1,611 us); in
+  // several waves the scan, with more warps to switch between, does (4 x 16 heads, Dk = 128: 3,037 us against 4,016).
+  if (Cf::GATE == 1 && (Cf::DK == 128 || (Cf::DK == 64 && Cf::J == 8)) && grid > sms) return -1000;
   if (grid <= 0 || grid > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
   // one block per SM anyway: four more warps take the preparation off the state warps
   const int prep = grid <= sms ? 4 : 0;

@@ -32,9 +32,12 @@ int pick(const LaunchArgs &a) {
     // Few heads: with 128 state values per lane their blocks would not fill the SMs and a warp would spend most of a token in
     // its own FMAs.  8 key dimensions per lane spread the state over 4 (J = 4) or 2 times as many warps.  The rule looks at
     // the whole problem and not at T: a prefill and the decode steps that continue it take the same split, hence the same bits.
+    // (AUTO promises those bits below 64 tokens only.  Its longer calls that end up here, with decays per key and Temporal priors, issue
+    // more than they wait: 8 x 16 heads, 2,048 tokens, 2,109 us as it is, 3,720 us with the finer split.)
+    const bool fine = a.algo != SWILA_ALGO_AUTO || a.p.T < 64;
     if constexpr ((J == 4 || J == 8) && GATE <= 1) {
       constexpr int WIDE = ScanCfg<IO, J, DK, 128, TB, GATE>::COLS;
-      if (a.algo != SWILA_ALGO_SCAN_WIDE && a.heads * ((a.p.Dv + WIDE - 1) / WIDE) < sm_count()) {
+      if (fine && a.heads * ((a.p.Dv + WIDE - 1) / WIDE) < sm_count()) {
         if (a.p.T == 1) return launch_scan<ScanCfg<IO, J, DK, DK, 1, GATE, 8>, POST>(a);
         return launch_scan<ScanCfg<IO, J, DK, DK, TB, GATE, 8>, POST>(a);
       }

@@ -730,7 +730,8 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
               again.prime(p, m, ln, gates_s, cols, wcol, tg, nvalid);
               tile_trip<Cf, true>(p, m, ln, again, P2, gk_s, cols + Cf::PAD, tg, nvalid, colr, tok);
             } else {
-              tile_trip_again<Cf>(&p, &m, xch, gates_s, gk_s, cols, wcol, tg, nvalid, colr, tok);
+              const TileSmem smem_copy = m;  // (a copy: the fast path's own may stay in registers)
+              tile_trip_again<Cf>(&p, &smem_copy, xch, gates_s, gk_s, cols, wcol, tg, nvalid, colr, tok);
               const int slots = tg == 0 ? C : 8;
 #pragma unroll
               for (int i = 0; i < RL; ++i)

@@ -42,10 +42,12 @@ def test_blocked_scan_matches_oracle(binding, oracle, w0, var):
     plain = gpu_forward(binding, w, dev)
     binding.device_status()
     assert_close(w, got, ref, w.name)
-    if binding.auto_algo(w, aux_outputs=False) == binding.ALGO_SCAN:
+    # auxiliary outputs or Temporal priors on top of decays are left to the sequential scan, as are operands that do not fit shared memory
+    left = w.gated and w.Dk >= 64 and w.J < 16
+    if not left and binding.auto_algo(w, aux_outputs=False) == binding.ALGO_SCAN:
         assert torch.equal(got["o"], plain["o"]) and torch.equal(got["W"], plain["W"])
     scan = gpu_forward(binding, w, dev, algo=binding.ALGO_SCAN)
-    if not (w.Dk == 128 and w.J == 16 and w.gated):
+    if not (w.Dk == 128 and w.J == 16 and w.gated) and not (left and w.temporal):
         assert not torch.equal(scan["W"], plain["W"])  # it was not the sequential scan that ran
 
 
