@@ -146,7 +146,7 @@ int swila_state_init(const swila_shape_t *shape, swila_state_t *state, void *str
  * SWILA_ERR_ALIAS: o, r_debug or a tensor of state_out overlaps a streamed input (q, k, v, a gate tensor),
  * or o overlaps r_debug or the state; state_out may alias state_in only tensor for tensor, exactly.
  *
- * Which kernel runs (shape->algo).  Two kernels evaluate the same recurrence and agree to rounding
+ * Which kernel runs (shape->algo).  Several kernels evaluate the same recurrence and agree to rounding
  * (1e-4 on the state):
  *   SCAN   the sequential scan on the FP32 ALUs: every shape, dtype, flag and output.
  *   CHUNK  32-token chunks whose state-times-token contractions run on the tcgen05 tensor cores (bf16
@@ -163,10 +163,13 @@ int swila_state_init(const swila_shape_t *shape, swila_state_t *state, void *str
  *              below 2^-40 (the chunked form divides by that product), which costs the scan's time.
  *          Requested for anything else (SWILA_GATE_PER_KEY and SWILA_GATE_ELEMENTWISE included: their decay
  *          differs per key dimension, so the rows of a tile share no operand): SWILA_ERR_UNSUPPORTED.
- *   AUTO   CHUNK when the call is inside that coverage and T >= 64, else SCAN.  So the following send an
- *          AUTO call to the scan kernel, at 3-6 times the cost per token: fp32 io, SWILA_QKV_ACT, Dk = 16,
- *          J in {1, 2}, T < 64, SWILA_GATED with per-key or elementwise decays or, at Dk = 128, with SWILA_TEMPORAL,
- *          and r_debug or statistics together with SWILA_GATED or J = 16.
+ *   AUTO   T < 64: SCAN.  T >= 64: CHUNK when the call is inside that coverage; else a block form of the
+ *          same recurrence at FP32 precision (16 tokens at a time on the tensor cores, every operand in three
+ *          bf16 parts, when ungated with Dk in {64, 128}; 4 or 8 tokens at a time on the FP32 ALUs with decays and at
+ *          Dk = 16); else SCAN.  The last is what remains for: SWILA_GATE_ELEMENTWISE; SWILA_GATED with
+ *          SWILA_TEMPORAL, r_debug or statistics at Dk in {64, 128} and J < 16; per-key decays at Dk = 128, or with J = 8,
+ *          when the heads fill more than one wave of SMs, and with J = 16 at Dk = 128.  The block forms equal
+ *          SCAN to rounding, not bit for bit: ask for SCAN where a prefill has to equal decode steps exactly.
  * Inside CHUNK the work distribution depends on state_out: with a state output, when the 128-row tiles
  * of the launch do not fill a whole number of waves of SMs, the chunk sequence is cut into equal runs
  * per SM and a tile that falls into two runs hands its state over through state_out (a cooperative
@@ -203,7 +206,8 @@ typedef struct {
 /*
  * swila_forward that also forms the sums of `stats` (which must not be NULL; any of its members may be).
  * The kernel is chosen as in swila_forward; outputs and state are those of swila_forward with the same
- * shape->algo, bit for bit.  The chunked kernel adds its sums with atomic operations (the pieces of a sequence
+ * shape->algo, bit for bit where the same kernel serves both (a SWILA_GATED call under AUTO may take another
+ * one for its statistics: to rounding then).  The chunked kernel adds its sums with atomic operations (the pieces of a sequence
  * may run in different thread blocks), so their last bits can differ from run to run; the scan kernel's do not.
  */
 int swila_forward_stats(const swila_shape_t *shape, const void *q, const void *k, const void *v,
