@@ -558,9 +558,9 @@ int launch_scan(const LaunchArgs &a) {
   const long long grid = nslice * a.p.B * a.p.H;
   if (grid <= 0 || grid > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;
   // Set up while the launch before it in the stream still runs (a decode step of a small model is as short as its own
-  // launch latency); the kernel starts with launch_wait.  Long calls are not: blocks placed early, beside those that still run,
-  // end up two to an SM while others idle, for as long as the kernel takes (1 x 16 heads, 2,048 tokens, J = 8, Dk = 128: 2,155 ->
-  // 2,529 us per call when calls follow each other).
+  // launch latency); the kernel starts with launch_wait.  Not where a call's blocks, placed early, would share SMs with those that
+  // still run: they end up two to an SM while others idle, for as long as the call takes (2 x 16 heads, 36 tokens, Dk = 64:
+  // 19.6 -> 30.7 us per call when calls follow each other).  A few tokens are over before that matters.
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
@@ -570,7 +570,7 @@ int launch_scan(const LaunchArgs &a) {
   cfg.dynamicSmemBytes = C::SMEM_BYTES;
   cfg.stream = a.stream;
   cfg.attrs = &attr;
-  cfg.numAttrs = a.p.T < 64 ? 1 : 0;
+  cfg.numAttrs = a.p.T <= 4 || (a.p.T < 64 && 2 * grid <= sm_count()) ? 1 : 0;
   e = cudaLaunchKernelEx(&cfg, kern, a.p);
   if (e != cudaSuccess) (void)cudaGetLastError();
   return (int)e;

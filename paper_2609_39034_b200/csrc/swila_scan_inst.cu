@@ -32,12 +32,13 @@ int pick(const LaunchArgs &a) {
     // Few heads: with 128 state values per lane their blocks would not fill the SMs and a warp would spend most of a token in
     // its own FMAs.  8 key dimensions per lane spread the state over 4 (J = 4) or 2 times as many warps.  The rule looks at
     // the whole problem and not at T: a prefill and the decode steps that continue it take the same split, hence the same bits.
-    // (AUTO promises those bits below 64 tokens only.  Its longer calls that end up here, with decays per key and Temporal priors, issue
-    // more than they wait: 8 x 16 heads, 2,048 tokens, 2,109 us as it is, 3,720 us with the finer split.)
-    const bool fine = a.algo != SWILA_ALGO_AUTO || a.p.T < 64;
+    // It pays while the wide blocks leave a third of the SMs idle (36 tokens, Dk = 128, J = 4: 24 heads 28.8 -> 28.7 us, 32 heads 28.8 ->
+    // 32.8; Dk = 64, 16 heads: 30.8 -> 20.5), and with eight components' per-key decays, whose staging leaves one block per SM, while
+    // the finer split is a single wave (Dk = 64, 32 heads: 48.2 -> 45.1 us, 64 heads: 49.2 -> 86.0).
     if constexpr ((J == 4 || J == 8) && GATE <= 1) {
-      constexpr int WIDE = ScanCfg<IO, J, DK, 128, TB, GATE>::COLS;
-      if (fine && a.heads * ((a.p.Dv + WIDE - 1) / WIDE) < sm_count()) {
+      constexpr int WIDE = ScanCfg<IO, J, DK, 128, TB, GATE>::COLS, FINE = ScanCfg<IO, J, DK, DK, TB, GATE, 8>::COLS;
+      const bool wave = !(GATE == 1 && J == 8) || a.heads * ((a.p.Dv + FINE - 1) / FINE) <= sm_count();
+      if (3 * a.heads * ((a.p.Dv + WIDE - 1) / WIDE) <= 2 * sm_count() && wave) {
         if (a.p.T == 1) return launch_scan<ScanCfg<IO, J, DK, DK, 1, GATE, 8>, POST>(a);
         return launch_scan<ScanCfg<IO, J, DK, DK, TB, GATE, 8>, POST>(a);
       }

@@ -92,6 +92,10 @@ struct TileMaps {
 };
 
 // ---- instructions ----------------------------------------------------------------------------
+__device__ __forceinline__ void tile_add(float (&a)[4], const float (&b)[4]) {
+#pragma unroll
+  for (int e = 0; e < 4; ++e) a[e] += b[e];  // (packed additions would tie register pairs: 782 -> 803 us for a layer of 32 heads, 3,000 tokens)
+}
 __device__ __forceinline__ void tile_mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
                : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
@@ -667,6 +671,8 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
             tile_split(w0[2], w0[3], q[1]);
             tile_split(w1[0], w1[1], q[2]);
             tile_split(w1[2], w1[3], q[3]);
+            // (fp32 results: each K step sums from zero, so that the tensor pipe's truncations do not add up in one long chain)
+            [[maybe_unused]] float d[4][4] = {};
 #pragma unroll
             for (int pa = Cf::NPW - 1; pa >= 0; --pa)
 #pragma unroll
@@ -674,8 +680,12 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
                 if (pa + s < Cf::NPW) {
                   const uint32_t a[4] = {q[0][pa], q[1][pa], q[2][pa], q[3][pa]};
 #pragma unroll
-                  for (int n = 0; n < 4; ++n) tile_mma(acc[x][n], a, bq[s][n >> 1][(n & 1) * 2], bq[s][n >> 1][(n & 1) * 2 + 1]);
+                  for (int n = 0; n < 4; ++n) tile_mma(Cf::ES == 4 ? d[n] : acc[x][n], a, bq[s][n >> 1][(n & 1) * 2], bq[s][n >> 1][(n & 1) * 2 + 1]);
                 }
+            if constexpr (Cf::ES == 4) {
+#pragma unroll
+              for (int n = 0; n < 4; ++n) tile_add(acc[x][n], d[n]);
+            }
           }
         }
 #pragma unroll
@@ -788,14 +798,19 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
             for (int s = 0; s < NPK; ++s)
 #pragma unroll
               for (int x = 0; x < 2; ++x) tile_ldsm_t(bk[s][x], (t3 ^ (((n4 + 2 * x) & 7) * 16)) + s * Cf::PART + (n4 >> 3) * 4096);
+            // The block's own sum first, added to the state on the FP32 ALUs: the tensor pipe truncates when it aligns a product with its
+            // accumulator, and truncations at the state's magnitude, all of one sign, would add up over the sequence.
+            float d[4][4] = {};
 #pragma unroll
             for (int pa = 2; pa >= 0; --pa)
 #pragma unroll
               for (int s = 0; s < NPK; ++s)
                 if (pa + s < 3) {
 #pragma unroll
-                  for (int n = 0; n < 4; ++n) tile_mma(w[mt][n4 + n], c[pa], bk[s][n >> 1][(n & 1) * 2], bk[s][n >> 1][(n & 1) * 2 + 1]);
+                  for (int n = 0; n < 4; ++n) tile_mma(d[n], c[pa], bk[s][n >> 1][(n & 1) * 2], bk[s][n >> 1][(n & 1) * 2 + 1]);
                 }
+#pragma unroll
+            for (int n = 0; n < 4; ++n) tile_add(w[mt][n4 + n], d[n]);
           }
         }
       }
