@@ -38,6 +38,10 @@ int block_dispatch_any(const LaunchArgs &a) {
     if (a.Dk == 128) return bf16 ? tile_dispatch<128, true>(a, err, sms) : tile_dispatch<128, false>(a, err, sms);
     return block_dispatch<16, 0>(a, err, sms);
   }
+  if (a.gate_mode == 1 && a.Dk == 64) {
+    const int rc = a.io_dtype == SWILA_IO_BF16 ? tile_dispatch<64, true>(a, err, sms) : tile_dispatch<64, false>(a, err, sms);
+    if (rc != -1000) return rc;
+  }
 #define SWILA_CASE(DK)                                                     \
   case DK:                                                                 \
     if (a.gate_mode == 1) return block_dispatch<DK, 1>(a, err, sms);       \

@@ -29,10 +29,11 @@
 
 namespace swila {
 
-template <typename IO_, int J_, int DK_, int MT_, bool EXT_, int NPK_>
+template <typename IO_, int J_, int DK_, int MT_, bool EXT_, int NPK_, bool GATED_ = false>
 struct TileCfg {
   using IO = IO_;
   static constexpr int J = J_, DK = DK_, MT = MT_, NPK = NPK_;
+  static constexpr bool GATED = GATED_;  // one decay per key dimension and component: operands of a component's own
   static constexpr bool EXT = EXT_;  // the instantiation with the Temporal priors, r_debug and the statistics
   static constexpr int C = 16;       // tokens per block: the K extent of one matrix instruction
   static constexpr int ES = (int)sizeof(IO);
@@ -48,10 +49,19 @@ struct TileCfg {
   static constexpr int NCS = CPW >= 8 ? CPW / 8 : 1, NCL = 2 * MT / NCS, GC = CPW >= 8 ? 8 : CPW;  // GC: columns among the 8 values of g
   static_assert(R % 32 == 0 && J * CPW == R && CL * OCL == RL && LPC * CL == J, "row split");
   static constexpr int PAD = 16 / ES;
-  static constexpr int NB = 3;                                        // ring of operand tiles
+  static constexpr int NB = GATED ? 1 : 3;                            // ring of operand tiles
+  static constexpr int MS = GATED ? 1 : 2;                            // row tiles at a time in the products with the state
+  static constexpr int OJ = GATED ? J : 1;                            // operand sets
+  // Gated: a row tile belongs to one component.  J / 2 warps then share GCOLS columns: in the products with the state each has two
+  // components of all of them, token by token each has all components of CPW of them; the exchange rows carry one to the other.
+  static constexpr int GW = GATED && J > 2 ? J / 2 : 1, GCOLS = CPW * GW;
+  static_assert(!GATED || (DK == 64 && MT == 2 && J <= 4 && NPK == 3 && !EXT), "");
   static constexpr int PART = (DK / 64) * 32 * 128;                   // one part of [k ; q] of a block: rows of 128 bytes, 128-byte swizzle
   static constexpr int RAWKQ = NPK == 1 ? 0 : 2 * C * DK * ES;        // k and q as they arrive, when they have to be converted
-  static constexpr int GK = C * 20 * 4;                               // k_s.k_t, fp32 rows of 20
+  static constexpr int NRAW = GATED ? 1 : 2;
+  static constexpr int UPART = C * 128;                               // Gated: one part of 16 vectors (k_t / A_t; k_t times the later decays)
+  static constexpr int ALPHA = GATED ? C * J * DK * 4 : 0;
+  static constexpr int GK = C * 20 * 4 + (GATED ? 16 : 0);                               // k_s.k_t, fp32 rows of 20
   static constexpr int GQP = C * 48;                                  // one part of k_s.q_t (s <= t) as [t][s] bf16, rows of 48 bytes
   // exchange rows of a warp, 7 units of 16 bytes (an odd number: the rows of a matrix load fall into different banks).  First
   // p_0 .. p_15 in units 0..3; then the coefficients' parts, of tokens 0..7 in units 0, 1, 4, of tokens 8..15 in units 2, 3, 5; then
@@ -64,7 +74,7 @@ struct TileCfg {
 __host__ __device__ constexpr int tile_up128(int n) { return (n + 127) & ~127; }
 
 struct TileSmem {
-  int kq, rawkq, gates, gates_stage, g_be, g_pk, g_pq, g_gk, g_gq, gk, gq, xch, wb, bars, total;
+  int kq, rawkq, kb, kh, alpha, ac, scale, gates, gates_stage, g_be, g_pk, g_pq, g_gk, g_gq, gk, gq, xch, wb, bars, total;
 };
 template <class Cf>
 __host__ __device__ inline TileSmem tile_smem(int nwarps, bool temporal, int gate_bufs) {
@@ -72,14 +82,19 @@ __host__ __device__ inline TileSmem tile_smem(int nwarps, bool temporal, int gat
   const int cols = nwarps * Cf::CPW, grow = cols + Cf::PAD;
   const int gate = tile_up128(Cf::C * Cf::J * grow * Cf::ES), vec = tile_up128(Cf::C * cols * Cf::ES);
   int off = 0;
-  m.kq = off; off += Cf::NB * Cf::NPK * Cf::PART;
-  m.rawkq = off; off += 2 * Cf::RAWKQ;
+  m.kq = off; off += Cf::NB * Cf::OJ * Cf::NPK * Cf::PART;
+  m.kb = off; off += Cf::GATED ? Cf::J * 3 * Cf::UPART : 0;
+  m.kh = off; off += Cf::GATED ? Cf::J * 3 * Cf::UPART : 0;
+  m.rawkq = off; off += Cf::NRAW * Cf::RAWKQ;
+  m.alpha = off; off += Cf::ALPHA;
+  m.ac = off; off += Cf::GATED ? Cf::J * Cf::DK * 4 : 0;
+  m.scale = off; off += Cf::GATED ? 128 : 0;
   m.gates = off;
   m.g_be = vec; m.g_pk = m.g_be + gate; m.g_pq = m.g_pk + gate; m.g_gk = m.g_pq + gate;
   m.g_gq = m.g_gk + (temporal ? vec : 0); m.gates_stage = m.g_gq + (temporal ? vec : 0);
   off += gate_bufs * m.gates_stage;
-  m.gk = off; off += 2 * Cf::GK;
-  m.gq = off; off += 2 * 3 * Cf::GQP;
+  m.gk = off; off += 2 * Cf::OJ * Cf::GK;
+  m.gq = off; off += 2 * Cf::OJ * 3 * Cf::GQP;
   m.xch = off; off += nwarps * Cf::XCH;
   m.wb = off; off += temporal ? nwarps * Cf::WB : 0;
   m.bars = off; off += 64;
@@ -88,7 +103,7 @@ __host__ __device__ inline TileSmem tile_smem(int nwarps, bool temporal, int gat
 }
 
 struct TileMaps {
-  CUtensorMap k, q, v, be, pk, pq, gk, gq;
+  CUtensorMap k, q, v, be, pk, pq, gk, gq, al;
 };
 
 // ---- instructions ----------------------------------------------------------------------------
@@ -194,44 +209,160 @@ __device__ __forceinline__ void tile_convert(const unsigned char *raw, unsigned 
   }
 }
 
-// Half of a Gram matrix of a block (8 of its 16 columns, n8) by one warp.  which = 0: k_s.k_t as fp32 rows [s][t] for the E-step; 1: k_s.q_t, zero for s > t, as
-// [t][s] in three bf16 parts, the B operand of the readouts.
-template <class Cf>
-__device__ __forceinline__ void tile_gram(const unsigned char *tile, int which, int n8, float *gk, unsigned char *gq, int lane) {
-  float d[4] = {0.f, 0.f, 0.f, 0.f};
-  const uint32_t base = umma::smem_u32(tile);
-  const int arow = (which ? 16 : 0) + (lane & 7) + ((lane >> 3) & 1) * 8, brow = n8 * 8 + (lane & 7);
-  uint32_t b[Cf::NPK][4];  // (a matrix load of B brings two K steps)
+// Half of a Gram matrix of a block (8 of its 16 columns, n8) by one warp.  which = 0: u_s.k_t as fp32 rows [s][t] for the E-step; 1:
+// u_s.q_t, zero for s > t, as [t][s] in bf16 parts, the B operand of the readouts.  The vectors k_t, q_t are the rows of `tile`, u_s those of
+// `us` (k_s itself, or k_s over the decays so far), whose parts are `upart` bytes apart.
+template <class Cf, int NH = 1>
+__device__ __forceinline__ void tile_gram(const unsigned char *tile, const unsigned char *us, int upart, int which, int n8, float *gk, unsigned char *gq, int lane) {
+  float d[NH][2][4] = {};  // two chains of matrix instructions each
+  const uint32_t abase = which ? umma::smem_u32(tile) + 16 * 128 : umma::smem_u32(us), bbase = which ? umma::smem_u32(us) : umma::smem_u32(tile);
+  const int apart = which ? Cf::PART : upart, bpart = which ? upart : Cf::PART;
+  const int arow = (lane & 7) + ((lane >> 3) & 1) * 8, brow = n8 * 8 + (lane & 7);
+  uint32_t b[NH][Cf::NPK][4];  // (a matrix load of B brings two K steps)
 #pragma unroll
   for (int ks = 0; ks < Cf::KS; ++ks) {
     uint32_t a[Cf::NPK][4];
 #pragma unroll
     for (int p = 0; p < Cf::NPK; ++p) {
-      tile_ldsm(a[p], base + p * Cf::PART + tile_at(arow, 2 * ks + (lane >> 4)));
-      if ((ks & 1) == 0) tile_ldsm(b[p], base + p * Cf::PART + tile_at(brow, 2 * ks + (lane >> 3)));
+      tile_ldsm(a[p], abase + p * apart + tile_at(arow, 2 * ks + (lane >> 4)));
+#pragma unroll
+      for (int n = 0; n < NH; ++n)
+        if ((ks & 1) == 0) tile_ldsm(b[n][p], bbase + p * bpart + tile_at(brow + n * 8, 2 * ks + (lane >> 3)));
     }
 #pragma unroll
     for (int pa = 0; pa < Cf::NPK; ++pa)
 #pragma unroll
       for (int pb = 0; pb < Cf::NPK; ++pb)
         if (pa + pb < 3) {
-          tile_mma(d, a[pa], b[pb][(ks & 1) * 2], b[pb][(ks & 1) * 2 + 1]);
+#pragma unroll
+          for (int n = 0; n < NH; ++n) tile_mma(d[n][pb & 1], a[pa], b[n][pb][(ks & 1) * 2], b[n][pb][(ks & 1) * 2 + 1]);
         }
   }
   const int g = lane >> 2, t2 = (lane & 3) * 2;
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int row = g + 8 * h, c = 8 * n8 + t2;
-    if (which == 0) {
-      *reinterpret_cast<float2 *>(gk + row * 20 + c) = make_float2(d[2 * h], d[2 * h + 1]);
-    } else {
-      uint32_t p[Cf::RPARTS];
-      tile_split(c <= row ? d[2 * h] : 0.f, c + 1 <= row ? d[2 * h + 1] : 0.f, p);
+  for (int n = 0; n < NH; ++n)
 #pragma unroll
-      for (int s = 0; s < Cf::RPARTS; ++s) *reinterpret_cast<uint32_t *>(gq + s * Cf::GQP + row * 48 + c * 2) = p[s];
+    for (int h = 0; h < 2; ++h) {
+      const int row = g + 8 * h, c = 8 * (n8 + n) + t2;
+      const float x = d[n][0][2 * h] + d[n][1][2 * h], y = d[n][0][2 * h + 1] + d[n][1][2 * h + 1];
+      if (which == 0) {
+        *reinterpret_cast<float2 *>(gk + row * 20 + c) = make_float2(x, y);
+      } else {
+        uint32_t p[Cf::RPARTS];
+        tile_split(c <= row ? x : 0.f, c + 1 <= row ? y : 0.f, p);
+#pragma unroll
+        for (int s = 0; s < Cf::RPARTS; ++s) *reinterpret_cast<uint32_t *>(gq + s * Cf::GQP + row * 48 + c * 2) = p[s];
+      }
+    }
+}
+
+// Gated, one block: per component, from the decays a_t and A_t = a_1 ... a_t, the vectors A_t k_t and A_t q_t of the products with the state (the
+// post-decay form of Eq. 3.7 predicts with A_{t-1}) and k_t / A_t for the Gram matrices, in three parts.  Returns whether some A is too
+// small for that quotient.  A thread takes one component and two key dimensions.
+template <class Cf>
+struct TileDecay {
+  const unsigned char *raw;
+  const float *alpha, *scale;  // scale: of the 32 vectors, when k and q are activated
+  bool act;
+  __device__ __forceinline__ float2 vec(int row, int d) const {  // rows 0..15: k, 16..31: q
+    const typename Cf::IO *src = reinterpret_cast<const typename Cf::IO *>(raw) + row * Cf::DK + d;
+    float2 x = make_float2(to_f32(src[0]), to_f32(src[1]));
+    if (act) {
+      const float sc = scale[row];
+      x = make_float2(silu_approx(x.x) * sc, silu_approx(x.y) * sc);
+    }
+    return x;
+  }
+  __device__ __forceinline__ float2 decay(int t, int j, int d, int nvalid) const {  // 1 past the end of the sequence
+    return t < nvalid ? *reinterpret_cast<const float2 *>(alpha + (t * Cf::J + j) * Cf::DK + d) : make_float2(1.f, 1.f);
+  }
+  static __device__ __forceinline__ void put(unsigned char *dst, int part_bytes, int row, int d, float2 x) {
+    uint32_t p[3];
+    tile_split(x.x, x.y, p);
+#pragma unroll
+    for (int s = 0; s < 3; ++s) *reinterpret_cast<uint32_t *>(dst + s * part_bytes + tile_at(row, d >> 3) + (d & 7) * 2) = p[s];
+  }
+};
+// Four tokens at a time: their operands are fetched before the stores, which the compiler does not move loads across.
+template <class Cf>
+__device__ __forceinline__ bool tile_decay(const TileDecay<Cf> &in, unsigned char *tile, unsigned char *kh, int nvalid, bool post, int j, int d) {
+  bool tiny = false;
+  unsigned char *tj = tile + j * 3 * Cf::PART, *hj = kh + j * 3 * Cf::UPART;
+  float2 A = make_float2(1.f, 1.f);
+#pragma unroll 1
+  for (int t0 = 0; t0 < Cf::C; t0 += 4) {
+    float2 k[4], q[4], a[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a[i] = in.decay(t0 + i, j, d, nvalid);
+      k[i] = in.vec(t0 + i, d);
+      q[i] = in.vec(16 + t0 + i, d);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float2 before = A;
+      A = mul2(A, a[i]);
+      in.put(tj, Cf::PART, t0 + i, d, mul2(post ? before : A, k[i]));
+      in.put(tj, Cf::PART, 16 + t0 + i, d, mul2(A, q[i]));
+      in.put(hj, Cf::UPART, t0 + i, d, make_float2(k[i].x * rcp_approx(A.x), k[i].y * rcp_approx(A.y)));
+      tiny = tiny || !(fminf(A.x, A.y) > 1e-18f && fmaxf(A.x, A.y) < 1e18f);
     }
   }
+  return tiny;
 }
+// ... and the update operand, k_t times the decays after t, with the product of all of them.
+template <class Cf>
+__device__ __forceinline__ void tile_decay_update(const TileDecay<Cf> &in, unsigned char *kb, float *ac, int nvalid, int j, int d) {
+  float2 S = make_float2(1.f, 1.f);
+#pragma unroll 1
+  for (int t0 = Cf::C - 4; t0 >= 0; t0 -= 4) {
+    float2 k[4], a[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a[i] = in.decay(t0 + i, j, d, nvalid);
+      k[i] = in.vec(t0 + i, d);
+    }
+#pragma unroll
+    for (int i = 3; i >= 0; --i) {
+      in.put(kb + j * 3 * Cf::UPART, Cf::UPART, t0 + i, d, mul2(S, k[i]));
+      S = mul2(S, a[i]);
+    }
+  }
+  *reinterpret_cast<float2 *>(ac + j * Cf::DK + d) = S;
+}
+// The Gram matrices with the decays multiplied out between s and t: exact for any decay, zero included.  Rare, so not optimised.
+template <class Cf>
+__device__ __noinline__ void tile_gram_products(const TileDecay<Cf> *in, float *gk, unsigned char *gq, int nvalid, bool post, int tid, int nt) {
+  constexpr int C = Cf::C;
+  for (int it = tid; it < Cf::J * C * C; it += nt) {
+    const int j = it / (C * C), s = (it / C) % C, t = it % C;
+    float2 dk = make_float2(0.f, 0.f), dq = dk;
+    if (t >= s) {
+      for (int d = 0; d < Cf::DK; d += 2) {
+        float2 x = in->vec(s, d), xk = x;
+        for (int m = s + 1; m <= t; ++m) {
+          xk = x;
+          x = mul2(x, in->decay(m, j, d, nvalid));
+        }
+        dk = fma2(post ? xk : x, in->vec(t, d), dk);
+        dq = fma2(x, in->vec(16 + t, d), dq);
+      }
+    }
+    gk[j * (Cf::GK / 4) + s * 20 + t] = dk.x + dk.y;
+    uint32_t p[3];
+    tile_split(dq.x + dq.y, 0.f, p);
+#pragma unroll
+    for (int n = 0; n < 3; ++n) *reinterpret_cast<unsigned short *>(gq + (j * 3 + n) * Cf::GQP + t * 48 + s * 2) = (unsigned short)p[n];
+  }
+}
+__device__ __forceinline__ int tile_bar_or(int id, int n, bool x) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %3, 0;\n\tbarrier.cta.red.or.pred q, %1, %2, p;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+      : "=r"(r) : "r"(id), "r"(n), "r"((unsigned)x) : "memory");
+  return r;
+}
+__device__ __forceinline__ void tile_bar_arrive(int id, int n) { asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(n) : "memory"); }
 
 // ---- the serial part of a block: RL rows per lane ------------------------------------------------
 template <class Cf>
@@ -344,15 +475,17 @@ __device__ __forceinline__ bool tile_trip(const ScanParams &p, const TileSmem &m
   auto P = [&](int r, int i) -> float & { return (i & 1) ? P2[r][i >> 1].y : P2[r][i >> 1].x; };
   bool bad = false;
   gk_s += tg * 84;  // row tg, column tg
-  float gk[C];      // k_t.k_t' of one token t with the slots of the window
+  constexpr int NG = Cf::GATED ? RL : 1;
+  float gk[NG][C];  // k_t.k_t' of one token t with the slots of the window (Gated: of each of the lane's components)
   auto push = [&](int i) {  // token tg + i into the slots from i + 2 on
 #pragma unroll
     for (int r = 0; r < RL; ++r) {
       const float cp = P(r, i);
       const float2 c2 = make_float2(cp, cp);
-      if (i & 1) P(r, i + 2) = fmaf(cp, gk[i + 2], P(r, i + 2));
+      const float(&gr)[C] = gk[r % NG];
+      if (i & 1) P(r, i + 2) = fmaf(cp, gr[i + 2], P(r, i + 2));
 #pragma unroll
-      for (int u = (i + 3) / 2; u < C / 2; ++u) P2[r][u] = fma2(c2, make_float2(gk[2 * u], gk[2 * u + 1]), P2[r][u]);
+      for (int u = (i + 3) / 2; u < C / 2; ++u) P2[r][u] = fma2(c2, make_float2(gr[2 * u], gr[2 * u + 1]), P2[r][u]);
     }
   };
 #pragma unroll
@@ -387,8 +520,11 @@ __device__ __forceinline__ bool tile_trip(const ScanParams &p, const TileSmem &m
         if (i > 0) push(i - 1);
 #pragma unroll
         for (int q = (i + 1) / 4; q < C / 4; ++q) {
-          const float4 y = tile_lds4(gk_s + i * 80 + q * 16);
-          gk[4 * q] = y.x; gk[4 * q + 1] = y.y; gk[4 * q + 2] = y.z; gk[4 * q + 3] = y.w;
+#pragma unroll
+          for (int n = 0; n < NG; ++n) {
+            const float4 y = tile_lds4(gk_s + (Cf::GATED ? (ln.comp0 + n % CL) * Cf::GK : 0) + i * 80 + q * 16);
+            gk[n][4 * q] = y.x; gk[n][4 * q + 1] = y.y; gk[n][4 * q + 2] = y.z; gk[n][4 * q + 3] = y.w;
+          }
         }
         gt.activate(t + 1 < nvalid, p.qkv_act, temporal);
         gt.fetch(m, grow, temporal);  // (two tokens past the block at its end: inside shared memory, unused)
@@ -413,7 +549,7 @@ __device__ __forceinline__ bool tile_trip(const ScanParams &p, const TileSmem &m
       }
     }
 #pragma unroll
-    for (int r = 0; r < RL; ++r) P(r, i + 1) = fmaf(P(r, i), gk[i + 1], P(r, i + 1));  // the push that the next token waits for
+    for (int r = 0; r < RL; ++r) P(r, i + 1) = fmaf(P(r, i), gk[r % NG][i + 1], P(r, i + 1));  // the push that the next token waits for
   }
   push(GT - 1);
   return bad;
@@ -431,7 +567,7 @@ __device__ __noinline__ void tile_trip_again(const ScanParams *p, const TileSmem
 #pragma unroll
   for (int i = 0; i < Cf::RL; ++i) ln.rp[i] = ln.rho[i] = ln.s_r[i] = ln.s_rh[i] = ln.s_q[i] = ln.s_qh[i] = 0.f;
   float2 P2[Cf::RL][Cf::C / 2];
-  auto row = [&](int i) { return reinterpret_cast<float2 *>(xch + ((ln.comp0 + i % Cf::CL) * Cf::CPW + ln.col + (i / Cf::CL) * Cf::LCOLS) * Cf::XROW + tg * 4); };
+  auto row = [&](int i) { return reinterpret_cast<float2 *>(xch + ((ln.comp0 + i % Cf::CL) * Cf::GCOLS + ln.col + (i / Cf::CL) * Cf::LCOLS) * Cf::XROW + tg * 4); };
   const int slots = tg == 0 ? Cf::C : 8;
 #pragma unroll
   for (int i = 0; i < Cf::RL; ++i)
@@ -489,7 +625,7 @@ __device__ __forceinline__ void tile_weights(const ScanParams &p, const TileSmem
 
 // ---- the kernel ---------------------------------------------------------------------------
 template <class Cf>
-__global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
+__global__ void __maxnreg__(Cf::MT * Cf::DK <= 128 ? 168 : 255)
     swila_tile_kernel(const __grid_constant__ ScanParams p, const __grid_constant__ TileMaps maps, const int nwarps, const int gate_bufs, int *err) {
   using IO = typename Cf::IO;
   using namespace umma;
@@ -515,6 +651,12 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
   ln.comp0 = (lane / Cf::LCOLS) * Cf::CL;
   ln.col = lane % Cf::LCOLS;
   const int wcol = warp * CPW;  // the warp's first column inside the slice
+  const int wg = warp % Cf::GW, gbase = (warp - wg) * CPW;  // its place in its group; the group's first column
+  auto comp_of = [&](int mt) { return Cf::GATED ? (J == 1 ? 0 : wg * 2 + mt) : 0; };
+  auto group_sync = [&]() {
+    if constexpr (Cf::GW > 1) named_bar_sync(5 + warp / Cf::GW, Cf::GW * 32);
+    else __syncwarp();
+  };
 #pragma unroll
   for (int r = 0; r < RL; ++r) {
     ln.rp[r] = ln.rho[r] = 1.0f / J;
@@ -528,7 +670,7 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
   }
 
   if (tid == 0) {
-    for (int i = 0; i < 3; ++i) mbar_init(&bars[i], 1);
+    for (int i = 0; i < 3; ++i) mbar_init(&bars[i], Cf::GATED ? 2 : 1);
     for (int i = 3; i < 5; ++i) mbar_init(&bars[i], nt >= 128 ? 4 : 1);  // the threads that issue the gates' copies
     mbar_fence_init();
   }
@@ -545,7 +687,11 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
         tma_load_3d(dst + hf * 4096 + 2048, &maps.q, hf * 64, b * C, bh, bar);
       }
     } else {
-      unsigned char *dst = smem + m.rawkq + (b & 1) * Cf::RAWKQ;
+      unsigned char *dst = smem + m.rawkq + (Cf::GATED ? 0 : b & 1) * Cf::RAWKQ;
+      if constexpr (Cf::GATED) {
+        mbar_arrive_expect_tx(bar, Cf::ALPHA);  // (the barrier counts two arrivals then)
+        tma_load_4d(smem + m.alpha, &maps.al, 0, 0, b * C, bh, bar);
+      }
       tma_load_3d(dst, &maps.k, 0, b * C, bh, bar);
       tma_load_3d(dst + Cf::RAWKQ / 2, &maps.q, 0, b * C, bh, bar);
     }
@@ -579,13 +725,79 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
   };
   if (ptid == 0) load_kq(0);
 
+  [[maybe_unused]] const int all = (int)blockDim.x;
+  if constexpr (Cf::GATED) {
+    // Preparation warps.  Iteration b: the update operand of block b first: it takes the place of block b-1's, which has been used.  Then block
+    // b+1: its vectors take the place of block b's once the state warps have formed their products.
+    if (!holds) {
+      const TileDecay<Cf> in{smem + m.rawkq, reinterpret_cast<const float *>(smem + m.alpha), reinterpret_cast<const float *>(smem + m.scale), p.qkv_act != 0};
+      float *scale = reinterpret_cast<float *>(smem + m.scale);
+      constexpr int PAIRS = J * DK / 2;
+#pragma unroll 1
+      for (int b = -1; b < nb; ++b) {
+        if (b >= 0) {
+          if (lane == 0) {
+            fence_async_smem();
+            load_gates(b, ptid >> 5, 4);
+          }
+#pragma unroll 1
+          for (int i = ptid; i < PAIRS; i += 128) {
+            const int j = i / (DK / 2), d = (i % (DK / 2)) * 2;
+            tile_decay_update<Cf>(in, smem + m.kb, reinterpret_cast<float *>(smem + m.ac), min(C, p.T - b * C), j, d);
+          }
+          named_bar_sync(1, 128);
+          tile_bar_arrive(3, all);
+        }
+        if (b + 1 < nb) {
+          if (ptid == 0 && b >= 0) {
+            fence_async_smem();
+            load_kq(b + 1);
+          }
+          const int nv1 = min(C, p.T - (b + 1) * C);
+          wait_kq(b + 1);
+          if (p.qkv_act) {
+            for (int i = ptid; i < 32 * (DK / 8); i += 128) {  // norms of the 32 vectors: 8 lanes each
+              const int row = i / (DK / 8), d = (i % (DK / 8)) * 8;
+              const IO *src = reinterpret_cast<const IO *>(in.raw) + row * DK + d;
+              float ss = 0.f;
+#pragma unroll
+              for (int n = 0; n < 8; ++n) { const float x = silu_approx(to_f32(src[n])); ss = fmaf(x, x, ss); }
+#pragma unroll
+              for (int off = 1; off < DK / 8; off <<= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+              if (i % (DK / 8) == 0) scale[row] = rsqrtf(ss + kL2Eps);
+            }
+            named_bar_sync(1, 128);
+          }
+          bool tiny = false;
+          if (b >= 0) named_bar_sync(2, all);
+#pragma unroll 1
+          for (int i = ptid; i < PAIRS; i += 128) tiny = tile_decay<Cf>(in, smem + m.kq, smem + m.kh, nv1, p.post, i / (DK / 2), (i % (DK / 2)) * 2) || tiny;
+          const int slow = tile_bar_or(1, 128, tiny);
+          float *gk1 = reinterpret_cast<float *>(smem + m.gk + ((b + 1) & 1) * J * Cf::GK);
+          unsigned char *gq1 = smem + m.gq + ((b + 1) & 1) * J * 3 * Cf::GQP;
+          if (slow) {
+            tile_gram_products<Cf>(&in, gk1, gq1, nv1, p.post, ptid, 128);
+          } else {
+#pragma unroll 1
+            for (int i = ptid >> 5; i < 2 * J; i += 4) {
+              const int jj = i >> 1;
+              tile_gram<Cf, 2>(smem + m.kq + jj * 3 * Cf::PART, smem + m.kh + jj * 3 * Cf::UPART, Cf::UPART, i & 1, 0, gk1 + jj * (Cf::GK / 4), gq1 + jj * 3 * Cf::GQP, lane);
+            }
+          }
+        }
+        named_bar_sync(4, all);
+      }
+      return;
+    }
+  }
+
   // ---- state -> accumulator tiles: tile (mt, n8), rows g and g + 8 of its 16, key dims 8 n8 + t2 + {0, 1} ----
   float w[MT][N8][4];
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int rho = mt * 16 + h * 8 + g, comp = rho / CPW, col = col0 + wcol + rho % CPW;
+      const int rho = mt * 16 + h * 8 + g, comp = Cf::GATED ? comp_of(mt) : rho / CPW, col = col0 + (Cf::GATED ? gbase + rho % Cf::GCOLS : wcol + rho % CPW);
       const float *src = (p.W_in && holds && col < p.Dv) ? p.W_in + (((size_t)bh * J + comp) * p.Dv + col) * DK : nullptr;
 #pragma unroll
       for (int n = 0; n < N8; ++n) {
@@ -598,8 +810,8 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
 
   // Iteration b: operands of block b+2 (converted, or on their way), Gram matrices of block b+1, then block b itself.
 #pragma unroll 1
-  for (int b = -2; b < nb; ++b) {
-    if (prepares && lane == 0) {
+  for (int b = Cf::GATED ? -1 : -2; b < nb; ++b) {
+    if (!Cf::GATED && prepares && lane == 0) {
       const int pwarp = ptid >> 5, parts = nt >= 128 ? 4 : 1;
       if (pwarp < parts) {
         fence_async_smem();
@@ -615,7 +827,7 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
         if (bg >= 0 && bg < nb) load_gates(bg, pwarp, parts);
       }
     }
-    if (prepares) {
+    if (!Cf::GATED && prepares) {
       if constexpr (NPK == 3) {
         if (b + 2 < nb) {
           wait_kq(b + 2);
@@ -627,16 +839,17 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
         const unsigned char *tile1 = smem + m.kq + ((b + 1) % Cf::NB) * NPK * Cf::PART;
         float *gk1 = reinterpret_cast<float *>(smem + m.gk + ((b + 1) & 1) * Cf::GK);
         unsigned char *gq1 = smem + m.gq + ((b + 1) & 1) * 3 * Cf::GQP;
-        for (int i = ptid >> 5; i < 4; i += nt >> 5) tile_gram<Cf>(tile1, i >> 1, i & 1, gk1, gq1, lane);
+        for (int i = ptid >> 5; i < 4; i += nt >> 5) tile_gram<Cf>(tile1, tile1, Cf::PART, i >> 1, i & 1, gk1, gq1, lane);
       }
     }
     if (holds && b >= 0) {
       const int nvalid = min(C, p.T - b * C);
       const unsigned char *gates = smem + m.gates + (gate_bufs == 2 ? b & 1 : 0) * m.gates_stage;
-      const float *gk = reinterpret_cast<const float *>(smem + m.gk + (b & 1) * Cf::GK);
+      const float *gk = reinterpret_cast<const float *>(smem + m.gk + (b & 1) * Cf::OJ * Cf::GK);
       const uint32_t tile = smem_u32(smem + m.kq + (b % Cf::NB) * NPK * Cf::PART);
-      const uint32_t gq = smem_u32(smem + m.gq + (b & 1) * 3 * Cf::GQP);
+      const uint32_t gq = smem_u32(smem + m.gq + (b & 1) * Cf::OJ * 3 * Cf::GQP);
       unsigned char *xch = smem + m.xch + warp * Cf::XCH;
+      unsigned char *xtok = smem + m.xch + (warp - wg) * Cf::XCH + wg * CPW * Cf::XROW;  // the rows of its columns
       float *wb = reinterpret_cast<float *>(smem + m.wb + warp * Cf::WB);
       if constexpr (NPK == 1) wait_kq(b);  // (completed before: it makes the copies visible to this thread)
 
@@ -645,12 +858,12 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
       const uint32_t t3 = tile + tile_at(((lane >> 3) & 1) * 8 + (lane & 7), lane >> 4);       // update, transposed
       const size_t tok = tok0 + (size_t)b * C;
       float r[MT][2][4];
-      // ---- p and r of the block: W (in parts) times the 32 vectors, two row tiles at a time ----
+      // ---- p and r of the block: W (in parts) times the 32 vectors, Cf::MS row tiles at a time ----
 #pragma unroll
-      for (int mp = 0; mp < MT; mp += 2) {
-        float acc[2][4][4];
+      for (int mp = 0; mp < MT; mp += Cf::MS) {
+        float acc[Cf::MS][4][4];
 #pragma unroll
-        for (int x = 0; x < 2; ++x)
+        for (int x = 0; x < Cf::MS; ++x)
 #pragma unroll
           for (int n = 0; n < 4; ++n)
 #pragma unroll
@@ -658,13 +871,16 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
 #pragma unroll
         for (int ks = 0; ks < KS; ++ks) {
           uint32_t bq[NPK][2][4];
+          auto operand = [&](int comp) {
 #pragma unroll
           for (int s = 0; s < NPK; ++s)
 #pragma unroll
             for (int x = 0; x < 2; ++x)
-              tile_ldsm(bq[s][x], (t1 ^ ((ks & 3) * 32)) + s * Cf::PART + x * 2048 + (ks >> 2) * 4096);
+              tile_ldsm(bq[s][x], comp * 3 * Cf::PART + (t1 ^ ((ks & 3) * 32)) + s * Cf::PART + x * 2048 + (ks >> 2) * 4096);
+          };
 #pragma unroll
-          for (int x = 0; x < 2; ++x) {
+          for (int x = 0; x < Cf::MS; ++x) {
+            if (x == 0) operand(comp_of(mp));
             const float(&w0)[4] = w[mp + x][2 * ks], (&w1)[4] = w[mp + x][2 * ks + 1];
             uint32_t q[4][Cf::NPW];
             tile_split(w0[0], w0[1], q[0]);
@@ -689,7 +905,7 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
           }
         }
 #pragma unroll
-        for (int x = 0; x < 2; ++x) {
+        for (int x = 0; x < Cf::MS; ++x) {
           unsigned char *xr = xch + ((mp + x) * 16 + g) * Cf::XROW + t2 * 4;
 #pragma unroll
           for (int n = 0; n < 2; ++n)
@@ -701,7 +917,10 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
             for (int e = 0; e < 4; ++e) r[mp + x][n][e] = acc[x][n + 2][e];
         }
       }
-      __syncwarp();
+      if constexpr (Cf::GATED) {
+        if (b + 1 < nb) tile_bar_arrive(2, all);  // the next block's vectors may take this one's place
+      }
+      group_sync();
 
       // ---- token by token, in two trips of eight.  Rolled: the loop over the blocks has to stay inside the instruction cache (with
       //      64 rows per warp and 16 tokens straight it is fetched at three quarters of the GPC cache's rate) ----
@@ -710,7 +929,7 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
         unsigned char *row[RL];
 #pragma unroll
         for (int i = 0; i < RL; ++i) {
-          row[i] = xch + ((ln.comp0 + i % Cf::CL) * CPW + ln.col + (i / Cf::CL) * Cf::LCOLS) * Cf::XROW;
+          row[i] = xtok + ((ln.comp0 + i % Cf::CL) * Cf::GCOLS + ln.col + (i / Cf::CL) * Cf::LCOLS) * Cf::XROW;
 #pragma unroll
           for (int q = 0; q < C / 4; ++q) {
             const float4 y = reinterpret_cast<const float4 *>(row[i])[q];
@@ -741,7 +960,7 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
               tile_trip<Cf, true>(p, m, ln, again, P2, gk_s, cols + Cf::PAD, tg, nvalid, colr, tok);
             } else {
               const TileSmem smem_copy = m;  // (a copy: the fast path's own may stay in registers)
-              tile_trip_again<Cf>(&p, &smem_copy, xch, gates_s, gk_s, cols, wcol, tg, nvalid, colr, tok);
+              tile_trip_again<Cf>(&p, &smem_copy, xtok, gates_s, gk_s, cols, wcol, tg, nvalid, colr, tok);
               const int slots = tg == 0 ? C : 8;
 #pragma unroll
               for (int i = 0; i < RL; ++i)
@@ -769,17 +988,36 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
         }
         if constexpr (Cf::EXT) tile_weights<Cf>(p, m, ln, gates, wb, cols, wcol, nvalid);
       }
-      __syncwarp();
+      group_sync();
 
       // ---- r += C (K Q^T masked), W += C K ----
       {
-        uint32_t bg[Cf::RPARTS][4];
+        if constexpr (Cf::GATED) {
+          named_bar_sync(3, all);  // the update operand is in place
+          const float *ac = reinterpret_cast<const float *>(smem + m.ac) + t2;
 #pragma unroll
-        for (int s = 0; s < Cf::RPARTS; ++s) tile_ldsm(bg[s], gq + s * Cf::GQP + (((lane >> 4) & 1) * 8 + (lane & 7)) * 48 + ((lane >> 3) & 1) * 16);
+          for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+            for (int n = 0; n < N8; ++n) {
+              const float2 a2 = *reinterpret_cast<const float2 *>(ac + comp_of(mt) * DK + n * 8);
+              const float2 lo = mul2(make_float2(w[mt][n][0], w[mt][n][1]), a2), hi = mul2(make_float2(w[mt][n][2], w[mt][n][3]), a2);
+              w[mt][n][0] = lo.x; w[mt][n][1] = lo.y; w[mt][n][2] = hi.x; w[mt][n][3] = hi.y;
+            }
+        }
+        // vectors of the update: 16 rows (tokens), transposed on the way to the registers
+        const uint32_t ut = Cf::GATED ? t3 - tile + smem_u32(smem + m.kb) : t3;
+        constexpr int UP = Cf::GATED ? Cf::UPART : Cf::PART;
+        uint32_t bg[Cf::RPARTS][4];
+        auto readout = [&](int comp) {
+#pragma unroll
+        for (int s = 0; s < Cf::RPARTS; ++s) tile_ldsm(bg[s], gq + (comp * 3 + s) * Cf::GQP + (((lane >> 4) & 1) * 8 + (lane & 7)) * 48 + ((lane >> 3) & 1) * 16);
+        };
         const uint32_t xa = smem_u32(xch) + ((lane & 7) + ((lane >> 3) & 1) * 8) * Cf::XROW;
         const int half = lane >> 4;
 #pragma unroll
         for (int mt = 0; mt < MT; ++mt) {
+          const int comp = comp_of(mt);
+          if (mt == 0 || Cf::GATED) readout(comp);
           uint32_t c[3][4];
 #pragma unroll
           for (int s = 0; s < 3; ++s) tile_ldsm(c[s], xa + mt * 16 * Cf::XROW + (half ? tile_c_at(s, 1) : tile_c_at(s, 0)));
@@ -797,7 +1035,7 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
 #pragma unroll
             for (int s = 0; s < NPK; ++s)
 #pragma unroll
-              for (int x = 0; x < 2; ++x) tile_ldsm_t(bk[s][x], (t3 ^ (((n4 + 2 * x) & 7) * 16)) + s * Cf::PART + (n4 >> 3) * 4096);
+              for (int x = 0; x < 2; ++x) tile_ldsm_t(bk[s][x], (ut ^ (((n4 + 2 * x) & 7) * 16)) + (comp * 3 + s) * UP + (n4 >> 3) * 4096);
             // The block's own sum first, added to the state on the FP32 ALUs: the tensor pipe truncates when it aligns a product with its
             // accumulator, and truncations at the state's magnitude, all of one sign, would add up over the sequence.
             float d[4][4] = {};
@@ -819,7 +1057,55 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
       //      NCL components each; with fewer than 8 columns per warp the other components are in lanes GC apart in g ----
       IO *ost = reinterpret_cast<IO *>(xch);
       __syncwarp();  // the coefficients have been read by all lanes
-      {
+      if constexpr (Cf::GATED) {
+        // (a lane's rows g and g + 8 of a tile are two columns of one component; each warp of a group finishes 16 / GW of the tokens)
+        const int grow = cols + Cf::PAD;
+        constexpr int SLOTS = Cf::GCOLS / 8;
+        const IO *const io = nullptr;
+        float val[2][2][SLOTS];
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+#pragma unroll
+            for (int cs = 0; cs < SLOTS; ++cs) {
+              if constexpr (J == 1) {
+                val[n][e][cs] = r[cs >> 1][n][(cs & 1) * 2 + e];
+              } else {
+                const uint32_t gpq = smem_u32(gates) + m.g_pq + ((8 * n + t2 + e) * J * grow + gbase + cs * 8 + g) * Cf::ES;
+                float x[J], mx, num = 0.f, den = 0.f;
+#pragma unroll
+                for (int c = 0; c < J; ++c) x[c] = tile_lds(gpq + c * grow * Cf::ES, io) * kLog2e;
+                mx = x[0];
+#pragma unroll
+                for (int c = 1; c < J; ++c) mx = fmaxf(mx, x[c]);
+#pragma unroll
+                for (int c = 0; c < J; ++c) {
+                  x[c] = ex2_approx(x[c] - mx);
+                  den += x[c];
+                }
+#pragma unroll
+                for (int mt = 0; mt < MT; ++mt) num = fmaf(Cf::GW > 1 && wg ? x[(J - 2 + mt) % J] : x[mt], r[mt][n][cs * 2 + e], num);
+                val[n][e][cs] = num * rcp_approx(den);
+              }
+            }
+        if constexpr (Cf::GW == 2) {
+          float4 *part = reinterpret_cast<float4 *>(xch + 1024);
+          part[lane] = wg ? make_float4(val[0][0][0], val[0][0][1], val[0][1][0], val[0][1][1]) : make_float4(val[1][0][0], val[1][0][1], val[1][1][0], val[1][1][1]);
+          group_sync();
+          const float4 y = *reinterpret_cast<const float4 *>(xch + (wg ? -Cf::XCH : Cf::XCH) + 1024 + lane * 16);
+          const float z[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i) from_f32(ost[(t2 + (i >> 1)) * Cf::GCOLS + (i & 1) * 8 + g], (wg ? val[1][i >> 1][i & 1] : val[0][i >> 1][i & 1]) + z[i]);
+        } else {
+#pragma unroll
+          for (int n = 0; n < 2; ++n)
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+#pragma unroll
+              for (int cs = 0; cs < SLOTS; ++cs) from_f32(ost[(8 * n + t2 + e) * Cf::GCOLS + cs * 8 + g], val[n][e][cs]);
+        }
+      } else {
         const int grow = cols + Cf::PAD;
         const int gcomp = g / Cf::GC, gcol = g % Cf::GC;
         const IO *const io = nullptr;
@@ -876,12 +1162,13 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
       }
       __syncwarp();
       {
-        constexpr int VB = CPW * Cf::ES < 16 ? CPW * Cf::ES : 16, VE = VB / Cf::ES, VPT = CPW / VE;
-        for (int i = lane; i < nvalid * VPT; i += 32) {
-          const int t = i / VPT, c = (i - t * VPT) * VE, col = col0 + wcol + c;
+        constexpr int GCOLS = Cf::GCOLS, VB = GCOLS * Cf::ES < 16 ? GCOLS * Cf::ES : 16, VE = VB / Cf::ES, VPT = GCOLS / VE;
+        const int t0 = wg * (C / Cf::GW);  // the warp's share of the tokens
+        for (int i = lane; i < min(C / Cf::GW, nvalid - t0) * VPT; i += 32) {
+          const int t = i / VPT, c = (i - t * VPT) * VE, col = col0 + gbase + c;
           if (col < p.Dv) {
-            IO *dst = (IO *)p.o + (tok + t) * p.Dv + col;
-            const IO *src = ost + t * CPW + c;
+            IO *dst = (IO *)p.o + (tok + t0 + t) * p.Dv + col;
+            const IO *src = ost + t * GCOLS + c;
             if constexpr (VB == 16) *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
             else if constexpr (VB == 8) *reinterpret_cast<uint2 *>(dst) = *reinterpret_cast<const uint2 *>(src);
             else *reinterpret_cast<uint32_t *>(dst) = *reinterpret_cast<const uint32_t *>(src);
@@ -889,7 +1176,8 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
         }
       }
     }
-    __syncthreads();
+    if constexpr (Cf::GATED) named_bar_sync(4, all);
+    else __syncthreads();
   }
 
   // ---- accumulator tiles -> state, carried distributions, statistics ----
@@ -897,7 +1185,7 @@ __global__ void __maxnreg__(Cf::MT *Cf::DK <= 128 ? 168 : 255)
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const int rho = mt * 16 + h * 8 + g, comp = rho / CPW, col = col0 + wcol + rho % CPW;
+      const int rho = mt * 16 + h * 8 + g, comp = Cf::GATED ? comp_of(mt) : rho / CPW, col = col0 + (Cf::GATED ? gbase + rho % Cf::GCOLS : wcol + rho % CPW);
       if (p.W_out && holds && col < p.Dv) {
         float *dst = p.W_out + (((size_t)bh * J + comp) * p.Dv + col) * DK;
 #pragma unroll
@@ -952,6 +1240,11 @@ bool tile_make_maps(const ScanParams &p, int cols, TileMaps *m) {
   bool ok = rows(&m->k, p.k, DK, kq_box, kq) && rows(&m->q, p.q, DK, kq_box, kq) && rows(&m->v, p.v, Dv, cols);
   ok = ok && gates(&m->be, p.beta_logit) && gates(&m->pk, p.pik_logit) && gates(&m->pq, p.piq_logit);
   if (p.temporal) ok = ok && rows(&m->gk, p.gk_logit, Dv, cols) && rows(&m->gq, p.gq_logit, Dv, cols);
+  if (Cf::GATED) {  // [BH][T][J][DK] fp32
+    const cuuint64_t dims[4] = {DK, J, T, BH}, strides[3] = {DK * 4, J * DK * 4, T * J * DK * 4};
+    const cuuint32_t box[4] = {(cuuint32_t)DK, (cuuint32_t)J, (cuuint32_t)Cf::C, 1};
+    ok = ok && tma_encode(&m->al, p.alpha, 4, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_DATA_TYPE_FLOAT32);
+  }
   return ok;
 }
 
@@ -964,16 +1257,23 @@ int tile_warps(const ScanParams &p, int sms) {
   while (nw < 4 && nw * Cf::CPW < p.Dv && 2 * nw * Cf::CPW + Cf::PAD <= 256) nw *= 2;
   while (nw > 1 && (nw / 2 * Cf::CPW) % 8 == 0 && bh * ((p.Dv + nw / 2 * Cf::CPW - 1) / (nw / 2 * Cf::CPW)) <= sms) nw /= 2;
   while ((nw * Cf::CPW) % 8 != 0) nw *= 2;
+  if constexpr (Cf::GATED) {
+    // The operands of every component leave one block per SM: as many warps as it can hold and the columns occupy, whole groups of them.
+    nw = Cf::GW;
+    while (nw < 8 && nw * Cf::CPW < p.Dv && 2 * nw * Cf::CPW + Cf::PAD <= 256 && tile_smem<Cf>(2 * nw, false, 1).total <= 227 * 1024) nw *= 2;
+    while (nw > Cf::GW && bh * ((p.Dv + nw / 2 * Cf::CPW - 1) / (nw / 2 * Cf::CPW)) <= sms) nw /= 2;
+  }
   return nw;
 }
 
 template <class Cf>
 int launch_tile(const LaunchArgs &a, int *err, int sms) {
-  const int nw = tile_warps<Cf>(a.p, sms), cols = nw * Cf::CPW;
+  const int nw = tile_warps<Cf>(a.p, sms);
+  const int cols = nw * Cf::CPW;
   const long long grid = (long long)a.p.B * a.p.H * ((a.p.Dv + cols - 1) / cols);
   // One block per SM or less: four more warps take the preparation off the state warps, and the gates are fetched a block ahead.
   // More blocks: they hide each other's waits, and shared memory decides how many are resident.
-  const int prep = grid <= sms ? 4 : 0, gate_bufs = grid <= sms ? 2 : 1;
+  const int prep = Cf::GATED || grid <= sms ? 4 : 0, gate_bufs = !Cf::GATED && grid <= sms ? 2 : 1;
   const TileSmem m = tile_smem<Cf>(nw, a.p.temporal != 0, gate_bufs);
   if (m.total > 227 * 1024) return -1000;
   if (grid <= 0 || grid > 0x7fffffffLL) return (int)cudaErrorInvalidConfiguration;

@@ -9,7 +9,7 @@
 namespace swila {
 
 namespace {
-template <int J, bool EXT, int NPK>
+template <int J, bool EXT, int NPK, bool GATED = false>
 int pick(const LaunchArgs &a, int *err, int sms) {
 #if SWILA_BF16
   using IO = __nv_bfloat16;
@@ -17,7 +17,7 @@ int pick(const LaunchArgs &a, int *err, int sms) {
   using IO = float;
 #endif
   // two row tiles per warp: 64 state registers per lane at Dk = 64, 128 at Dk = 128
-  return launch_tile<TileCfg<IO, J, SWILA_DK, 2, EXT, NPK>>(a, err, sms);
+  return launch_tile<TileCfg<IO, J, SWILA_DK, 2, EXT, NPK, GATED>>(a, err, sms);
 }
 template <bool EXT>
 int pick_j(const LaunchArgs &a, int *err, int sms) {
@@ -43,6 +43,15 @@ int pick_j(const LaunchArgs &a, int *err, int sms) {
 template <>
 int tile_dispatch<SWILA_DK, (SWILA_BF16 != 0)>(const LaunchArgs &a, int *err, int sms) {
   const bool ext = a.p.temporal || a.p.r_debug || a.p.r_sum || a.p.r_ent || a.p.rho_sum || a.p.rho_ent;
+  if (a.gate_mode == 1) {
+#if SWILA_DK == 64
+    if (ext) return -1000;
+    if (a.J == 1) return pick<1, false, 3, true>(a, err, sms);
+    if (a.J == 2) return pick<2, false, 3, true>(a, err, sms);
+    if (a.J == 4) return pick<4, false, 3, true>(a, err, sms);
+#endif
+    return -1000;
+  }
   return ext ? pick_j<true>(a, err, sms) : pick_j<false>(a, err, sms);
 }
 
