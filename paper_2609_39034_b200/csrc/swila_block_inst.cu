@@ -14,6 +14,8 @@ int pick(const LaunchArgs &a, int *err, int sms) {
   constexpr int DK = SWILA_DK, GATE = SWILA_GATE;
   if constexpr (GATE == 1 && DK == 128 && J == 16) {
     return -1000;  // the decayed operands of 16 components do not fit shared memory
+  } else if constexpr (GATE == 1 && DK == 64 && J <= 4) {
+    return -1000;  // the register-tile kernel's, or the scan's
   } else if constexpr (EXT && J < 16 && (DK == 64 || (DK == 128 && GATE == 2))) {
     // Temporal priors and statistics on top of the decays leave too few registers for the blocked loop: the scan is faster (8 x 16 heads,
     // 2,048 tokens, Dk = 64, per key: 2,109 us against 3,029; 2 x 16, Dk = 128, per output: 1,884 against 2,274)
