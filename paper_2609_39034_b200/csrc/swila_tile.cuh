@@ -265,9 +265,19 @@ struct TileDecay {
   const float *alpha, *scale;  // scale: of the 32 vectors, when k and q are activated
   bool act;
   __device__ __forceinline__ float2 vec(int row, int d) const {  // rows 0..15: k, 16..31: q
-    const typename Cf::IO *src = reinterpret_cast<const typename Cf::IO *>(raw) + row * Cf::DK + d;
-    float2 x = make_float2(to_f32(src[0]), to_f32(src[1]));
-    if (act) {
+    return act ? vec<true>(row, d) : vec<false>(row, d);
+  }
+  template <bool ACT>
+  __device__ __forceinline__ float2 vec(int row, int d) const {
+    const unsigned char *src = raw + (row * Cf::DK + d) * Cf::ES;
+    float2 x;
+    if constexpr (Cf::ES == 2) {
+      const uint32_t u = *reinterpret_cast<const uint32_t *>(src);
+      x = make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+    } else {
+      x = *reinterpret_cast<const float2 *>(src);
+    }
+    if constexpr (ACT) {
       const float sc = scale[row];
       x = make_float2(silu_approx(x.x) * sc, silu_approx(x.y) * sc);
     }
@@ -284,7 +294,7 @@ struct TileDecay {
   }
 };
 // Four tokens at a time: their operands are fetched before the stores, which the compiler does not move loads across.
-template <class Cf>
+template <class Cf, bool ACT>
 __device__ __forceinline__ bool tile_decay(const TileDecay<Cf> &in, unsigned char *tile, unsigned char *kh, int nvalid, bool post, int j, int d) {
   bool tiny = false;
   unsigned char *tj = tile + j * 3 * Cf::PART, *hj = kh + j * 3 * Cf::UPART;
@@ -295,8 +305,8 @@ __device__ __forceinline__ bool tile_decay(const TileDecay<Cf> &in, unsigned cha
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       a[i] = in.decay(t0 + i, j, d, nvalid);
-      k[i] = in.vec(t0 + i, d);
-      q[i] = in.vec(16 + t0 + i, d);
+      k[i] = in.template vec<ACT>(t0 + i, d);
+      q[i] = in.template vec<ACT>(16 + t0 + i, d);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -311,7 +321,7 @@ __device__ __forceinline__ bool tile_decay(const TileDecay<Cf> &in, unsigned cha
   return tiny;
 }
 // ... and the update operand, k_t times the decays after t, with the product of all of them.
-template <class Cf>
+template <class Cf, bool ACT>
 __device__ __forceinline__ void tile_decay_update(const TileDecay<Cf> &in, unsigned char *kb, float *ac, int nvalid, int j, int d) {
   float2 S = make_float2(1.f, 1.f);
 #pragma unroll 1
@@ -320,7 +330,7 @@ __device__ __forceinline__ void tile_decay_update(const TileDecay<Cf> &in, unsig
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       a[i] = in.decay(t0 + i, j, d, nvalid);
-      k[i] = in.vec(t0 + i, d);
+      k[i] = in.template vec<ACT>(t0 + i, d);
     }
 #pragma unroll
     for (int i = 3; i >= 0; --i) {
@@ -743,7 +753,8 @@ __global__ void __maxnreg__(Cf::MT * Cf::DK <= 128 ? 168 : 255)
 #pragma unroll 1
           for (int i = ptid; i < PAIRS; i += 128) {
             const int j = i / (DK / 2), d = (i % (DK / 2)) * 2;
-            tile_decay_update<Cf>(in, smem + m.kb, reinterpret_cast<float *>(smem + m.ac), min(C, p.T - b * C), j, d);
+            if (p.qkv_act) tile_decay_update<Cf, true>(in, smem + m.kb, reinterpret_cast<float *>(smem + m.ac), min(C, p.T - b * C), j, d);
+            else tile_decay_update<Cf, false>(in, smem + m.kb, reinterpret_cast<float *>(smem + m.ac), min(C, p.T - b * C), j, d);
           }
           named_bar_sync(1, 128);
           tile_bar_arrive(3, all);
@@ -771,7 +782,11 @@ __global__ void __maxnreg__(Cf::MT * Cf::DK <= 128 ? 168 : 255)
           bool tiny = false;
           if (b >= 0) named_bar_sync(2, all);
 #pragma unroll 1
-          for (int i = ptid; i < PAIRS; i += 128) tiny = tile_decay<Cf>(in, smem + m.kq, smem + m.kh, nv1, p.post, i / (DK / 2), (i % (DK / 2)) * 2) || tiny;
+          for (int i = ptid; i < PAIRS; i += 128) {
+            const int j = i / (DK / 2), d = (i % (DK / 2)) * 2;
+            const bool x = p.qkv_act ? tile_decay<Cf, true>(in, smem + m.kq, smem + m.kh, nv1, p.post, j, d) : tile_decay<Cf, false>(in, smem + m.kq, smem + m.kh, nv1, p.post, j, d);
+            tiny = tiny || x;
+          }
           const int slow = tile_bar_or(1, 128, tiny);
           float *gk1 = reinterpret_cast<float *>(smem + m.gk + ((b + 1) & 1) * J * Cf::GK);
           unsigned char *gq1 = smem + m.gq + ((b + 1) & 1) * J * 3 * Cf::GQP;
