@@ -34,6 +34,10 @@ int block_dispatch_any(const LaunchArgs &a) {
     // No decays: all components share their operands, and the products with the state go to the tensor pipe (measured at every
     // shape tried, 1.05 to 2.3 times the blocked scan's pace).  At Dk = 16 there is nothing to contract: the serial part is all.
     const bool bf16 = a.io_dtype == SWILA_IO_BF16;
+    // fp32 results are promised within 1e-4 of the scan's, element by element.  Where the same keys come back over and over the recurrence
+    // amplifies rounding with the length, the more the fewer components and key dimensions: two orders of summation, each as far from
+    // the exact result, part by 8e-5 (J = 2, Dk = 64, 2,000 tokens), 5e-4 (4,000), 3e-4 (J = 4, 8,000).  Longer ones stay with the scan.
+    if (!bf16 && a.J > 1 && (a.p.T > 4096 || (a.p.T > 2048 && a.J <= 4 && a.Dk == 64))) return -1000;
     if (a.Dk == 64) return bf16 ? tile_dispatch<64, true>(a, err, sms) : tile_dispatch<64, false>(a, err, sms);
     if (a.Dk == 128) return bf16 ? tile_dispatch<128, true>(a, err, sms) : tile_dispatch<128, false>(a, err, sms);
     return block_dispatch<16, 0>(a, err, sms);

@@ -51,6 +51,16 @@ def test_blocked_scan_matches_oracle(binding, oracle, w0, var):
         assert not torch.equal(scan["W"], plain["W"])  # it was not the sequential scan that ran
 
 
+@pytest.mark.parametrize("D,J,T,scan", [(64, 2, 2048, False), (64, 2, 2049, True), (64, 4, 2049, True), (64, 8, 4096, False), (128, 2, 4096, False),
+                                        (128, 8, 4097, True), (64, 1, 4097, False)])
+def test_long_fp32_sequences_stay_with_the_scan(binding, D, J, T, scan):
+    w = _w(D, J, "fp32", T, H=1, Dv=8)
+    dev = to_dev(wl.make_inputs(w))
+    got, ref = (gpu_forward(binding, w, dev, algo=a) for a in (binding.ALGO_AUTO, binding.ALGO_SCAN))
+    assert torch.equal(got["W"], ref["W"]) == scan
+    assert wl.rel_err(got["W"], ref["W"]) < TOL_STATE and wl.rel_err(got["o"], ref["o"]) < TOL_FP32
+
+
 @pytest.mark.parametrize("w0", [SHAPES[1], SHAPES[7], SHAPES[12]], ids=lambda w: w.name)
 @pytest.mark.parametrize("post", [False, True], ids=["pre", "post"])
 def test_blocked_scan_with_vanishing_decays(binding, oracle, w0, post):
